@@ -246,10 +246,10 @@ __device__ __forceinline__ void face3_frame(const Desc3& d, CellNT3<R>& L, R tau
     const R uw2 = wside >= 0 ? Cst<P>::uw(d, wside, a2) : R(0);
     if constexpr (SCH == 1) {
         face_flux3_tlbfs<R>(L, Rc, Tz + tauL, fl, keep, uw1, uw2, F);
-    } else if constexpr (sizeof(R) == 4) {  // FP32: the node stage in packed pairs
-        R O[5], Pn[3][2][5], En[3][4][5];
-        face3_nodes_f32(L, Rc, fl, O, Pn, En);
-        face_flux3_nodes<R>(O, Pn, En, Tz + tauL, fl, keep, uw1, uw2, F);
+    } else if constexpr (sizeof(R) == 4) {  // FP32: the column stage in packed pairs
+        Cols3<R> c;
+        face3_columns_f32(L, Rc, fl, c);
+        face_flux3_columns<R>(c, Tz + tauL, fl, keep, uw1, uw2, F);
     } else {
         face_flux3<R>(L, Rc, Tz + tauL, fl, keep, uw1, uw2, F);
     }
@@ -553,9 +553,12 @@ __global__ void __launch_bounds__(TX* TY) step3_kernel(const Desc3* __restrict__
             const R rho = one + dr;
             const R dtc = Cst<P>::dt(d);
             R src[3];
+            const R rbg = rho * Cst<P>::beta_g(d), dTr = T - Cst<P>::T_ref(d);
 #pragma unroll
-            for (int a = 0; a < 3; ++a) src[a] = rho * Cst<P>::force(d, a);
-            src[d.g_axis] = vfma(rho * Cst<P>::beta_g(d), T - Cst<P>::T_ref(d), src[d.g_axis]);
+            for (int a = 0; a < 3; ++a) {  // selected by value: no local-memory copy of src
+                src[a] = rho * Cst<P>::force(d, a);
+                src[a] = a == d.g_axis ? vfma(rbg, dTr, src[a]) : src[a];
+            }
             const R inv = P::rcp(rho - div[0]);
             R du[3], u1[3];
 #pragma unroll
