@@ -47,7 +47,8 @@ struct CellNT3 {
 //   e*    = e - 1/2 sum_a (Tbar d_a m_a + d_a (m_a tau)) + cs2/2 sum_a dd_a e
 // with m_a = rho u_a, X_ab = m_a u_b + cs2 drho delta_ab, e = rho T - Tbar.
 // keep = 1 on an interior face, 0 on a wall face whose tangential velocity
-// is (uw1, uw2): no mass through the wall, (rho u_t)* = rho* u_wall,t.
+// is (uw1, uw2), 0 on an interior face: no mass through the wall,
+// (rho u_t)* = rho* u_wall,t.
 // F = (mass, n-, t1-, t2-momentum, energy) flux along +n.
 //
 // The products are never formed node by node.  On a column they are
@@ -56,7 +57,7 @@ struct CellNT3 {
 //   d_t f   = 2 (odd part in t at a = 0),  dd_t f = 2 (t^2 coefficient),
 //   dd_t1t2 f = 4 (b c coefficient),
 //   dd_nt f = 2 (odd part in t on a = +1, minus that on a = -1):
-// the same numbers with a third fewer operations (286 a face against 435
+// the same numbers with a third fewer operations (284 a face against 435
 // for products at the 19 nodes), and without the cancellation of the node
 // differences.  FP64 runs at the FMA rate, so there the step follows the
 // count: 20 steps of an 80^3 mesh and the download, FP64, 34.8 -> 29.5 ms;
@@ -223,9 +224,8 @@ __host__ __device__ __forceinline__ void face_flux3_columns(const Cols3<V>& c, V
     const V rho_s = one + drs;
     // wall faces: no mass through the wall, the wall's tangential velocity
     ms[0] = ms[0] * keep;
-    const V wallr = (one - keep) * rho_s;
-    ms[1] = vfma(keep, ms[1], wallr * uw1);
-    ms[2] = vfma(keep, ms[2], wallr * uw2);
+    ms[1] = vfma(keep, ms[1], rho_s * uw1);
+    ms[2] = vfma(keep, ms[2], rho_s * uw2);
     const V inv = T::rcp(rho_s);
     const V un_s = ms[0] * inv;
     const V taus = (es - drs * Tbar) * inv;  // T* - Tbar

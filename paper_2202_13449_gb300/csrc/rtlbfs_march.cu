@@ -306,9 +306,9 @@ march_kernel(const CavityDesc* __restrict__ descs, CavityRun* __restrict__ runs,
             {
                 R F[4];
                 if constexpr (sizeof(R) == 4) {  // FP32: packed column stage
-                    R A[4], Sa[4], M[4], Sm[4], B[4], Sb[4];
-                    face_columns_f32<true>(vxl, vxr, gxxl, gyxl, gxxr, gyxr, flx, A, Sa, M, Sm, B, Sb);
-                    face_flux_columns<R>(A, Sa, M, Sm, B, Sb, Tz + vxl.w, flx, wsx >= 0 ? R(0) : R(1),
+                    R A[4], Sa[4], M[4], D[4], B[4], Sb[4];
+                    face_columns_f32<true>(vxl, vxr, gxxl, gyxl, gxxr, gyxr, flx, A, Sa, M, D, B, Sb);
+                    face_flux_columns<R>(A, Sa, M, D, B, Sb, Tz + vxl.w, flx, wsx >= 0 ? R(0) : R(1),
                                          wsx >= 0 ? P::bcU(dp, wsx) : R(0), F);
                 } else {
                     CellNT<R> L = {{vxl.x, vxl.y, vxl.z, R(0)}, {gxxl.x, gxxl.y, gxxl.z, gxxl.w},
@@ -325,9 +325,9 @@ march_kernel(const CavityDesc* __restrict__ descs, CavityRun* __restrict__ runs,
                 const int ws = (wall_s && jf == 0) ? kSideS : ((wall_n && jf == ny) ? kSideN : -1);
                 R F[4];
                 if constexpr (sizeof(R) == 4) {
-                    R A[4], Sa[4], M[4], Sm[4], B[4], Sb[4];
-                    face_columns_f32<false>(vyl, vyr, gyyl, gxyl, gyyr, gxyr, fly, A, Sa, M, Sm, B, Sb);
-                    face_flux_columns<R>(A, Sa, M, Sm, B, Sb, Tz + vyl.w, fly, ws >= 0 ? R(0) : R(1),
+                    R A[4], Sa[4], M[4], D[4], B[4], Sb[4];
+                    face_columns_f32<false>(vyl, vyr, gyyl, gxyl, gyyr, gxyr, fly, A, Sa, M, D, B, Sb);
+                    face_flux_columns<R>(A, Sa, M, D, B, Sb, Tz + vyl.w, fly, ws >= 0 ? R(0) : R(1),
                                          ws >= 0 ? P::bcU(dp, ws) : R(0), F);
                 } else {
                     CellNT<R> L = {{vyl.x, vyl.z, vyl.y, R(0)}, {gyyl.x, gyyl.z, gyyl.y, gyyl.w},
