@@ -246,9 +246,10 @@ int rtlbfs_set_scheme(rtlbfs_t h, int scheme);
 
 /*
  * Execution schedule of the step (results are the same up to FP rounding
- * order): kernel 0 = warp-marching strips (each warp walks a 28-column strip
- * up a chunk of chunk_rows rows, rolling its stencil window in registers;
- * chunk_rows 0 = chosen from the GPU size), kernel 1 = shared-memory tiles
+ * order; without this call a handle of one mesh picks its kernel by size):
+ * kernel 0 = warp-marching strips (each warp walks a strip of 60 columns, 28
+ * in FP64, up a chunk of chunk_rows rows, rolling its stencil window in
+ * registers; chunk_rows 0 = chosen from the GPU size), kernel 1 = shared-memory tiles
  * of 32 columns by chunk_rows rows (16, 14, 12, 10, 8, 4 or 2 in FP32; 16,
  * 8, 4 or 2 in FP64; 0 = the height whose tile count fills the SMs most
  * evenly), kernel 2 = the same tiles in one persistent cooperative launch
@@ -272,7 +273,7 @@ int rtlbfs_debug_withhold_tile(rtlbfs_t h, int tile);
 /*
  * Autotuner: time every candidate schedule (the tile kernel at each tile
  * height, the persistent tile kernel at each height it can take, and the
- * marching kernel with 8..256 rows per unit) for `steps` steps each on a
+ * marching kernel with several numbers of rows per unit) for `steps` steps each on a
  * device-side snapshot of the current state, restore the state exactly
  * (fields, step counter, residual) and keep the fastest schedule.  Writes
  * the choice and its time per step if the pointers are non-null.  Needs

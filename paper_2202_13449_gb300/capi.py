@@ -413,7 +413,7 @@ class Solver:
         shared-memory tiles (chunk_rows = tile height: 16, 14, 12, 10, 8, 4 or
         2 in FP32; 16, 8, 4 or 2 in FP64), 2: the same tiles in a persistent
         launch (one cavity whose tiles all fit at once); chunk_rows 0 picks
-        automatically."""
+        automatically.  Without this call the kernel is picked by size."""
         self._check(lib().rtlbfs_set_schedule(self._h, int(kernel), int(chunk_rows)),
                     "set_schedule")
 

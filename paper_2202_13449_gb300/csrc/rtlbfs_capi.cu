@@ -76,6 +76,7 @@ int rtlbfs_create_mesh(int nx, int ny, const double* xf, const double* yf, int p
         delete h;
         return RTLBFS_ERR_OOM;
     }
+    h->eng->choose_kernel_by_size();
     int rc = h->eng->init();
     if (rc == RTLBFS_OK) rc = h->eng->add(nx, ny, xf, yf, &h->slot);
     if (rc == RTLBFS_OK) rc = h->eng->set_conduction_state(h->slot);

@@ -248,26 +248,27 @@ __host__ __device__ __forceinline__ void mirror_grad_c(int kind, R nx, R ny, R g
 // (u_t, T) in packed FP32x2 instructions.
 __device__ __forceinline__ void face_columns_nt_f32(const rtlbfs::CellNT<float>& L, const rtlbfs::CellNT<float>& Rc,
                                                     const FaceLine<float>& fl, float A[4],
-                                                    float Sa[4], float M[4], float D[4],
+                                                    float Na[4], float M[4], float D[4],
                                                     float B[4], float Sb[4])
 {
     const float h = fl.h;
     const float wL = fl.cL + h, mwR = fl.cR - h;
     const float2 cL2 = make_float2(fl.cL, fl.cL), cR2 = make_float2(fl.cR, fl.cR);
     const float2 wL2 = make_float2(wL, wL), mwR2 = make_float2(mwR, mwR);
-    const float2 h2 = make_float2(h, h), half2 = make_float2(0.5f, 0.5f);
+    const float2 h2 = make_float2(h, h), mh2 = make_float2(-h, -h), half2 = make_float2(0.5f, 0.5f);
+    const float2 m1 = make_float2(-1.0f, -1.0f);
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
         const int k = 2 * i;
         const float2 ql = make_float2(L.q[k], L.q[k + 1]), qr = make_float2(Rc.q[k], Rc.q[k + 1]);
         const float2 nl = make_float2(L.gn[k], L.gn[k + 1]), nr = make_float2(Rc.gn[k], Rc.gn[k + 1]);
         const float2 tl = make_float2(L.gt[k], L.gt[k + 1]), tr = make_float2(Rc.gt[k], Rc.gt[k + 1]);
-        const float2 a = __ffma2_rn(nl, cL2, ql), sa = __fmul2_rn(tl, h2);
+        const float2 a = __ffma2_rn(nl, cL2, ql), na = __fmul2_rn(tl, mh2);
         const float2 b = __ffma2_rn(nr, cR2, qr), sb = __fmul2_rn(tr, h2);
         const float2 m = __fmul2_rn(half2, __fadd2_rn(__ffma2_rn(nl, wL2, ql), __ffma2_rn(nr, mwR2, qr)));
-        const float2 d = __fadd2_rn(sa, sb);
+        const float2 d = __ffma2_rn(na, m1, sb);
         A[k] = a.x, A[k + 1] = a.y;
-        Sa[k] = sa.x, Sa[k + 1] = sa.y;
+        Na[k] = na.x, Na[k + 1] = na.y;
         B[k] = b.x, B[k + 1] = b.y;
         Sb[k] = sb.x, Sb[k + 1] = sb.y;
         M[k] = m.x, M[k + 1] = m.y;
@@ -325,9 +326,9 @@ __host__ __device__ __forceinline__ void face_c(const R vL[4], const R gL[8], co
     constexpr bool packed = false;
 #endif
     if constexpr (packed) {
-        R A[4], Sa[4], M[4], D[4], B[4], Sb[4];
-        face_columns_nt_f32(L, Rr, fl, A, Sa, M, D, B, Sb);
-        face_flux_columns<R>(A, Sa, M, D, B, Sb, Tz + tauL, fl, keep, uwt, F);
+        R A[4], Na[4], M[4], D[4], B[4], Sb[4];
+        face_columns_nt_f32(L, Rr, fl, A, Na, M, D, B, Sb);
+        face_flux_columns<R>(A, Na, M, D, B, Sb, Tz + tauL, fl, keep, uwt, F);
     } else {
         face_flux<R>(L, Rr, Tz + tauL, fl, keep, uwt, F);
     }
@@ -1516,6 +1517,7 @@ namespace rtlbfs {
 template <>
 struct vtraits<rtlbfsc::CntC> {
     static rtlbfsc::CntC bc(double c) { return {c, c == 0.0}; }
+    static rtlbfsc::CntC neg(rtlbfsc::CntC x) { return {-x.v, x.zero}; }  // free
     static rtlbfsc::CntC rcp(rtlbfsc::CntC x)
     {
         ++rtlbfsc::g_tc.sfu;

@@ -237,13 +237,10 @@ __device__ __forceinline__ float fast_rcp(float x) { return __fdividef(1.0f, x);
 // -------------------------------------------------------------------------
 // Value types of the face arithmetic.  float / double: one face.  f2: two
 // faces at once in the packed FP32x2 instructions of sm_100+ (one issue
-// slot for two round-to-nearest FP32 operations); d2: the FP64 pair.
+// slot for two round-to-nearest FP32 operations).
 // -------------------------------------------------------------------------
 struct f2 {
     float x, y;
-};
-struct d2 {
-    double x, y;
 };
 
 __device__ __forceinline__ f2 mk(float2 v) { return {v.x, v.y}; }
@@ -256,10 +253,6 @@ __device__ __forceinline__ f2 operator-(f2 a, f2 b)
 __device__ __forceinline__ f2 operator*(f2 a, f2 b) { return mk(__fmul2_rn(fl2(a), fl2(b))); }
 __device__ __forceinline__ f2 vfma(f2 a, f2 b, f2 c) { return mk(__ffma2_rn(fl2(a), fl2(b), fl2(c))); }
 
-__host__ __device__ __forceinline__ d2 operator+(d2 a, d2 b) { return {a.x + b.x, a.y + b.y}; }
-__host__ __device__ __forceinline__ d2 operator-(d2 a, d2 b) { return {a.x - b.x, a.y - b.y}; }
-__host__ __device__ __forceinline__ d2 operator*(d2 a, d2 b) { return {a.x * b.x, a.y * b.y}; }
-__device__ __forceinline__ d2 vfma(d2 a, d2 b, d2 c) { return {fma(a.x, b.x, c.x), fma(a.y, b.y, c.y)}; }
 __device__ __forceinline__ float vfma(float a, float b, float c) { return fmaf(a, b, c); }
 __device__ __forceinline__ double vfma(double a, double b, double c) { return fma(a, b, c); }
 
@@ -269,21 +262,20 @@ template <>
 struct vtraits<float> {
     static __device__ __forceinline__ float bc(double c) { return (float)c; }
     static __device__ __forceinline__ float rcp(float x) { return __fdividef(1.0f, x); }
+    static __host__ __device__ __forceinline__ float neg(float x) { return -x; }
 };
 template <>
 struct vtraits<double> {
     static __device__ __forceinline__ double bc(double c) { return c; }
     static __device__ __forceinline__ double rcp(double x) { return 1.0 / x; }
+    static __host__ __device__ __forceinline__ double neg(double x) { return -x; }
 };
 template <>
 struct vtraits<f2> {
     static __device__ __forceinline__ f2 bc(double c) { return {(float)c, (float)c}; }
     static __device__ __forceinline__ f2 rcp(f2 x) { return {__fdividef(1.0f, x.x), __fdividef(1.0f, x.y)}; }
-};
-template <>
-struct vtraits<d2> {
-    static __device__ __forceinline__ d2 bc(double c) { return {c, c}; }
-    static __device__ __forceinline__ d2 rcp(d2 x) { return {1.0 / x.x, 1.0 / x.y}; }
+    // a packed operand has no sign modifier: one instruction
+    static __device__ __forceinline__ f2 neg(f2 x) { return x * f2{-1.0f, -1.0f}; }
 };
 
 // -------------------------------------------------------------------------
@@ -300,7 +292,7 @@ struct CellNT {
 };
 
 // Eqs. 29, 46-48 and the braces of Eqs. 57-59 for one face (V = float,
-// double) or two faces (V = f2, d2).  Output F = (mass, normal momentum,
+// double) or two faces (V = f2).  Output F = (mass, normal momentum,
 // tangential momentum, energy) flux through the face along +n, with the
 // constant c_s^2 dropped from the normal momentum flux (see the file
 // comment).  keep = 1 on an interior face, 0 on a wall face, whose
@@ -332,17 +324,19 @@ struct CellNT {
 // FP32 512^2 11.46 -> 11.26 ms for 1000 steps.)
 //
 // The first stage, face_columns, forms the column coefficients: values A, M,
-// B of the four primitives on a = -1, 0, +1, their slopes Sa, Sb on a = -1,
-// +1 (not the temperature's, which enter nowhere) and the doubled mean
-// slopes D; face_flux_columns does the rest.  u_wall is 0 on interior faces.
+// B of the four primitives on a = -1, 0, +1, the negated slopes Na on a =
+// -1 and the slopes Sb on a = +1 (not the temperature's, which enter
+// nowhere) and the doubled mean slopes D; face_flux_columns does the rest.
+// (The negated left slopes make the differences plain sums: a packed
+// operand has no sign modifier.)  u_wall is 0 on interior faces.
 template <typename V>
 __host__ __device__ __forceinline__ void face_columns(const CellNT<V>& L, const CellNT<V>& Rc,
-                                                      const FaceLine<V>& fl, V A[4], V Sa[4],
+                                                      const FaceLine<V>& fl, V A[4], V Na[4],
                                                       V M[4], V D[4], V B[4], V Sb[4])
 {
     using T = vtraits<V>;
     const V half = T::bc(0.5);
-    const V h = fl.h;
+    const V h = fl.h, mh = T::neg(h);
     const V wL = fl.cL + h, mwR = fl.cR - h;  // wL, -wR
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
@@ -350,24 +344,24 @@ __host__ __device__ __forceinline__ void face_columns(const CellNT<V>& L, const 
         B[k] = vfma(Rc.gn[k], fl.cR, Rc.q[k]);
         M[k] = half * (vfma(L.gn[k], wL, L.q[k]) + vfma(Rc.gn[k], mwR, Rc.q[k]));
         if (k < 3) {
-            Sa[k] = L.gt[k] * h;
+            Na[k] = L.gt[k] * mh;
             Sb[k] = Rc.gt[k] * h;
-            D[k] = Sa[k] + Sb[k];
+            D[k] = Sb[k] - Na[k];
         } else {
             D[k] = h * (L.gt[k] + Rc.gt[k]);
         }
     }
 }
 
-template <typename V>
-__host__ __device__ __forceinline__ void face_flux_columns(const V A[4], const V Sa[4], const V M[4],
-                                                           const V D[4], const V B[4],
-                                                           const V Sb[4], V Tbar,
-                                                           const FaceLine<V>& fl, V keep, V u_wall,
-                                                           V F[4])
+// wall(mn, mt, rho): the wall rule on the predicted (rho u_n)*, (rho u_t)*.
+template <typename V, class W>
+__host__ __device__ __forceinline__ void face_flux_wall(const V A[4], const V Na[4], const V M[4],
+                                                        const V D[4], const V B[4], const V Sb[4],
+                                                        V Tbar, const FaceLine<V>& fl, W wall,
+                                                        V F[4])
 {
     using T = vtraits<V>;
-    const V zero = T::bc(0.0), one = T::bc(1.0), three = T::bc(3.0);
+    const V one = T::bc(1.0), three = T::bc(3.0);
     const V half = T::bc(0.5), quarter = T::bc(0.25), m2 = T::bc(-2.0), mhalf = T::bc(-0.5);
     const V cs2 = T::bc(1.0 / 3.0), hcs2 = T::bc(0.5 / 3.0), mhcs2 = T::bc(-0.5 / 3.0);
     // centres (b = 0) of the three columns: rho u_n, rho u_t, products
@@ -391,14 +385,15 @@ __host__ __device__ __forceinline__ void face_flux_columns(const V A[4], const V
     const V Qt_o2 = vfma(D[3], mt_s, mt_l2 * TM);                          // rho u_t T: odd part
     // columns a = -1, +1: odd parts in b and their differences (d_xy / 2)
     const V rA = one + A[0], rB = one + B[0];
-    const V mnA_o = vfma(rA, Sa[1], Sa[0] * A[1]), mnB_o = vfma(rB, Sb[1], Sb[0] * B[1]);
-    const V mtA_o = vfma(rA, Sa[2], Sa[0] * A[2]);
-    const V dmt_o = vfma(rB, Sb[2], vfma(Sb[0], B[2], zero - mtA_o));
-    const V PntA_o = vfma(Sa[2], vfma(Sa[0], Sa[1], mnA), mnA_o * A[2]);
-    const V dPnt_o = vfma(Sb[2], vfma(Sb[0], Sb[1], mnB), vfma(mnB_o, B[2], zero - PntA_o));
+    const V nmnA_o = vfma(rA, Na[1], Na[0] * A[1]), mnB_o = vfma(rB, Sb[1], Sb[0] * B[1]);
+    const V nmtA_o = vfma(rA, Na[2], Na[0] * A[2]);
+    const V dmt_o = vfma(rB, Sb[2], vfma(Sb[0], B[2], nmtA_o));
+    const V nPntA_o = vfma(Na[2], vfma(Na[0], Na[1], mnA), nmnA_o * A[2]);
+    const V dPnt_o = vfma(Sb[2], vfma(Sb[0], Sb[1], mnB), vfma(mnB_o, B[2], nPntA_o));
     // differences along the normal (b = 0)
     const V dx_mn = mnB - mnA, dx_mt = mtB - mtA, dx_e = eB - eA, dx_dr = B[0] - A[0];
-    const V dx_Pnt = vfma(mnB, B[2], zero - mnA * A[2]), dx_Q = vfma(mnB, TB, zero - mnA * TA);
+    const V nmnA = T::neg(mnA);
+    const V dx_Pnt = vfma(mnB, B[2], nmnA * A[2]), dx_Q = vfma(mnB, TB, nmnA * TA);
     const V dxx_mn = vfma(m2, mnM, mnB + mnA), dxx_mt = vfma(m2, mtM, mtB + mtA);
     const V dxx_e = vfma(m2, eM, eB + eA), dxx_dr = vfma(m2, M[0], B[0] + A[0]);
     const V dxx_Pnn = vfma(m2, PnnM, PnnB + PnnA);
@@ -409,37 +404,51 @@ __host__ __device__ __forceinline__ void face_flux_columns(const V A[4], const V
     // Eq. 47: (rho u_n)*, (rho u_t)*
     V mns_ = vfma(hcs2, vfma(three, dxx_mn, vfma(half, mn_q4, dmt_o)),
                   vfma(mhalf, vfma(cs2, dx_dr, PnnB - PnnA) + Pnt_o2, mnM));
-    V mts_ = vfma(hcs2, vfma(T::bc(1.5), mt_q4, dxx_mt + (mnB_o - mnA_o)),
+    V mts_ = vfma(hcs2, vfma(T::bc(1.5), mt_q4, dxx_mt + (mnB_o + nmnA_o)),
                   vfma(mhalf, dx_Pnt + Ptt_o2, vfma(mhcs2, D[0], mtM)));
     // Eq. 48: (rho T)* - Tbar
     const V es_ = vfma(hcs2, vfma(half, e_q4, dxx_e), vfma(mhalf, dx_Q + Qt_o2, eM));
 
     const V rho_s = one + drs;
-    // wall faces: no mass through the wall, the wall's tangential velocity
-    mns_ = mns_ * keep;
-    mts_ = vfma(keep, mts_, rho_s * u_wall);
+    wall(mns_, mts_, rho_s);
     const V inv = T::rcp(rho_s);
     const V uns = mns_ * inv, uts = mts_ * inv;
-    const V as_ = (es_ - drs * Tbar) * inv;  // T* - Tbar
+    const V as_ = vfma(drs, T::neg(Tbar), es_) * inv;  // T* - Tbar
 
     // Eqs. 57-59 braces along the face normal; d_y f = 2 (odd part)
     F[0] = mns_;
     const V Xnn0 = vfma(cs2, M[0], PnnM);
     F[1] = vfma(fl.m_nu_2h, vfma(three, dx_mn, mt_l2),
                 vfma(fl.m_tf15, vfma(mns_, uns, cs2 * drs) - Xnn0, Xnn0));
-    F[2] = vfma(fl.m_nu_2h, mn_l2 + dx_mt, vfma(fl.m_tf15, vfma(mns_, uts, zero - PntM), PntM));
+    F[2] = vfma(fl.m_nu_2h, mn_l2 + dx_mt, vfma(fl.m_tf15, vfma(mns_, uts, T::neg(PntM)), PntM));
     // (rho u_n T)* - (rho u_n T)^n = Tbar (mn* - mn0) + mn* a* - mn0 a0
     F[3] = vfma(fl.m_chi_2h, dx_e,
-                vfma(fl.m_tg15, vfma(Tbar, mns_ - mnM, vfma(mns_, as_, zero - mnM * M[3])), QnM));
+                vfma(fl.m_tg15, vfma(Tbar, mns_ - mnM, vfma(mns_, as_, T::neg(mnM) * M[3])), QnM));
+}
+
+template <typename V>
+__host__ __device__ __forceinline__ void face_flux_columns(const V A[4], const V Na[4], const V M[4],
+                                                           const V D[4], const V B[4],
+                                                           const V Sb[4], V Tbar,
+                                                           const FaceLine<V>& fl, V keep, V u_wall,
+                                                           V F[4])
+{
+    // wall faces: no mass through the wall, the wall's tangential velocity
+    face_flux_wall<V>(A, Na, M, D, B, Sb, Tbar, fl,
+                      [&](V& mn, V& mt, V rho) {
+                          mn = mn * keep;
+                          mt = vfma(keep, mt, rho * u_wall);
+                      },
+                      F);
 }
 
 template <typename V>
 __host__ __device__ __forceinline__ void face_flux(const CellNT<V>& L, const CellNT<V>& Rc, V Tbar,
                                           const FaceLine<V>& fl, V keep, V u_wall, V F[4])
 {
-    V A[4], Sa[4], M[4], D[4], B[4], Sb[4];
-    face_columns<V>(L, Rc, fl, A, Sa, M, D, B, Sb);
-    face_flux_columns<V>(A, Sa, M, D, B, Sb, Tbar, fl, keep, u_wall, F);
+    V A[4], Na[4], M[4], D[4], B[4], Sb[4];
+    face_columns<V>(L, Rc, fl, A, Na, M, D, B, Sb);
+    face_flux_columns<V>(A, Na, M, D, B, Sb, Tbar, fl, keep, u_wall, F);
 }
 
 // Green-Gauss gradients of a cell p from its four neighbours in the
@@ -503,14 +512,15 @@ __device__ __forceinline__ void face_columns_f32(const Vec4<float>& vl, const Ve
                                                  const Vec4<float>& gnl, const Vec4<float>& gtl,
                                                  const Vec4<float>& gnr, const Vec4<float>& gtr,
                                                  const FaceLine<float>& fl, float A[4],
-                                                 float Sa[4], float M[4], float D[4], float B[4],
+                                                 float Na[4], float M[4], float D[4], float B[4],
                                                  float Sb[4])
 {
     const float h = fl.h;
     const float wL = fl.cL + h, mwR = fl.cR - h;
     const float2 cL2 = make_float2(fl.cL, fl.cL), cR2 = make_float2(fl.cR, fl.cR);
     const float2 wL2 = make_float2(wL, wL), mwR2 = make_float2(mwR, mwR);
-    const float2 h2 = make_float2(h, h), half2 = make_float2(0.5f, 0.5f);
+    const float2 h2 = make_float2(h, h), mh2 = make_float2(-h, -h), half2 = make_float2(0.5f, 0.5f);
+    const float2 m1 = make_float2(-1.0f, -1.0f);
     // the left cell's temperature is carried by Tbar = Tz + T_L
     const float2 ql[2] = {make_float2(vl.x, vl.y), make_float2(vl.z, 0.0f)};
     const float2 qr[2] = {make_float2(vr.x, vr.y), make_float2(vr.z, vr.w - vl.w)};
@@ -518,15 +528,15 @@ __device__ __forceinline__ void face_columns_f32(const Vec4<float>& vl, const Ve
     const float2 tl[2] = {make_float2(gtl.x, gtl.y), make_float2(gtl.z, gtl.w)};
     const float2 nr[2] = {make_float2(gnr.x, gnr.y), make_float2(gnr.z, gnr.w)};
     const float2 tr[2] = {make_float2(gtr.x, gtr.y), make_float2(gtr.z, gtr.w)};
-    float2 a[2], sa[2], m[2], d2[2], b[2], sb[2];
+    float2 a[2], na[2], m[2], d2[2], b[2], sb[2];
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
         a[i] = __ffma2_rn(nl[i], cL2, ql[i]);
-        sa[i] = __fmul2_rn(tl[i], h2);
+        na[i] = __fmul2_rn(tl[i], mh2);
         b[i] = __ffma2_rn(nr[i], cR2, qr[i]);
         sb[i] = __fmul2_rn(tr[i], h2);
         m[i] = __fmul2_rn(half2, __fadd2_rn(__ffma2_rn(nl[i], wL2, ql[i]), __ffma2_rn(nr[i], mwR2, qr[i])));
-        d2[i] = __fadd2_rn(sa[i], sb[i]);
+        d2[i] = __ffma2_rn(na[i], m1, sb[i]);
     }
     // face-frame order: (rho, u_n, u_t, T)
     auto put = [](const float2* v, float* d) {
@@ -536,7 +546,7 @@ __device__ __forceinline__ void face_columns_f32(const Vec4<float>& vl, const Ve
         d[3] = v[1].y;
     };
     put(a, A);
-    put(sa, Sa);
+    put(na, Na);
     put(m, M);
     put(d2, D);
     put(b, B);
@@ -662,7 +672,6 @@ __host__ __device__ __forceinline__ int wall_parity(int kind, int k)
 struct StoreD {
     using S = double;
     using R = double;
-    using V2 = d2;
     static __host__ __device__ __forceinline__ R val(S s, int) { return s; }
     static __host__ __device__ __forceinline__ R diff(S a, S b, int) { return a - b; }
     static __host__ __device__ __forceinline__ S add(S s, R d, int) { return s + d; }
@@ -695,7 +704,6 @@ struct StoreD {
 struct StoreQ {
     using S = int;
     using R = float;
-    using V2 = f2;
     // scale of quantity k: 2^-32 (rho - 1), 2^-31 (u, v), 2^-30 (T)
     static __host__ __device__ __forceinline__ double scale_d(int k)
     {

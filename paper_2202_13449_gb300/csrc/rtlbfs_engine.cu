@@ -586,6 +586,7 @@ int Engine::set_scheme(int scheme)
             if (c.active) c.dirty = true;  // the scheme lives in the descriptor
     }
     if (scheme_ == kSchemeTLBFS) {  // tile kernel, default height
+        auto_kernel_ = false;
         kernel_ = 1;
         chunk_rows_ = kTileYDefault;
     }
@@ -597,15 +598,20 @@ int Engine::set_kernel(int kind)
     if (kind < 0 || kind > 2) return fail(RTLBFS_ERR_ARG, "kernel kind must be 0, 1 or 2");
     if (scheme_ == kSchemeTLBFS && kind != 1)
         return fail(RTLBFS_ERR_ARG, "the TLBFS face stage runs on the tile kernel (1)");
-    if (kind != kernel_) {
-        kernel_ = kind;
-        tiles_dirty_ = true;
-        if (gexec_) {
-            cudaGraphExecDestroy(gexec_);
-            gexec_ = nullptr;
-        }
-    }
+    auto_kernel_ = false;
+    use_kernel(kind);
     return RTLBFS_OK;
+}
+
+void Engine::use_kernel(int kind)
+{
+    if (kind == kernel_) return;
+    kernel_ = kind;
+    tiles_dirty_ = true;
+    if (gexec_) {
+        cudaGraphExecDestroy(gexec_);
+        gexec_ = nullptr;
+    }
 }
 
 int Engine::set_chunk_rows(int rows)
@@ -626,33 +632,94 @@ int Engine::set_chunk_rows(int rows)
 // about ceil(tiles / SMs) deep on the busiest SM, and a tile of height h
 // costs its faces and gradient ring plus a fixed share (loads, barriers,
 // the residual), in face-equivalents: 65 h + 32 + 0.25 * 34 (h + 2) + 300.
-int Engine::pick_tile_height() const
+// FP32 leaves out heights below 8: one or two warps a block pass through a
+// tile's phases too slowly even when every tile has an SM of its own (64^2:
+// 10.0 us per step at h = 2, 7.0 at 4, 6.6 at 8, 6.7 at 14).  FP64 counts a
+// 16-row tile 1.17 times: one such block fills an SM's registers and its
+// phases overlap with nothing (400^2: 228 us at h = 16, 194 at 8).
+int Engine::pick_tile_height(double* us) const
 {
     if (scheme_ == kSchemeTLBFS) return kTileYDefault;
     int best_h = kTileYDefault;
     double best = 1e300;
+    long long best_deep = 1;
     for (int h : kTileHeights) {
         if (!tile_height_ok(precision_, h)) continue;
+        if (precision_ == RTLBFS_FP32 && h < 8) continue;
         long long tiles = 0;
         for (int s = 0; s < capacity_; ++s)
             if (slots_[s].active)
                 tiles += (long long)((slots_[s].nx + kTileX - 1) / kTileX) *
                          ((slots_[s].ny + h - 1) / h);
-        const double deep = (double)((tiles + sms_ - 1) / std::max(sms_, 1));
-        const double cost = deep * (65.0 * h + 32.0 + 0.25 * 34.0 * (h + 2) + 300.0);
+        const long long deep = (tiles + sms_ - 1) / std::max(sms_, 1);
+        double cost = (double)deep * (65.0 * h + 32.0 + 0.25 * 34.0 * (h + 2) + 300.0);
+        if (precision_ == RTLBFS_FP64 && h == 16) cost *= 1.17;
         if (cost < best * (1.0 - 1e-9)) {
             best = cost;
             best_h = h;
+            best_deep = deep;
         }
     }
+    if (us) {
+        // FP32 step time: 14-row tiles (cost 1378) one deep take 6.7 us, two
+        // 8.4, three 10.5, four (a full SM) 10.9, then 2.65 us a tile
+        const double f = best / (1378.0 * (double)best_deep);
+        *us = std::max(4.7 + (0.3 + 1.6 * (double)best_deep) * f, 2.65 * (double)best_deep * f);
+    }
+    return best_h;
+}
+
+// Rows per unit of the FP32 marching kernel: a warp passes H + 3.5 rows (the
+// chunk and its prologue) in about max(1.32, 1 + 0.105 w) us a row when w
+// warps share the SM (measured: 1.32 us at 4, 1.86 at 8, 2.2 at 12).  Units
+// beyond a full wave of 12 warps per SM run in further waves.
+int Engine::pick_march_rows(double* us) const
+{
+    const long long slots = (long long)sms_ * std::max(occ_march_, 1);
+    auto row_us = [](double w) { return std::max(1.32, 1.0 + 0.105 * w); };
+    int best_h = 16, maxny = 1;
+    double best = 1e300;
+    for (int s = 0; s < capacity_; ++s)
+        if (slots_[s].active) maxny = std::max(maxny, slots_[s].ny);
+    for (int H = 4; H <= 64; ++H) {
+        long long units = 0;
+        for (int s = 0; s < capacity_; ++s)
+            if (slots_[s].active)
+                units += (long long)((slots_[s].nx + kStrip2 - 1) / kStrip2) *
+                         ((slots_[s].ny + H - 1) / H);
+        const long long waves = units / slots, rest = units % slots;
+        double t = (double)waves * row_us((double)occ_march_);
+        if (rest) t += row_us((double)((rest + sms_ - 1) / sms_));
+        t *= H + 3.5;
+        if (t < best * (1.0 - 1e-9)) {
+            best = t;
+            best_h = H;
+        }
+        if (H >= maxny) break;
+    }
+    if (us) *us = best + 3.5;
     return best_h;
 }
 
 int Engine::rebuild_tiles()
 {
     std::vector<int4> t;
+    // A single cavity, unless a schedule was set: FP32 marches where that is modelled faster
+    // (from about 0.7 M cells: 1024^2 36.3, 4096^2 351 us per step
+    // against the tiles' 42 and 557; 512^2 18.2 against 10.9), FP64 takes tiles
+    // (64^2: 29 us against 269 in 16-row chunks, a serial chain of 20 rows).
+    // A batch marches: its cavities come and go, and a kernel that followed
+    // the mix would change a cavity's rounding on the way.
+    if (auto_kernel_) {
+        double tile_us = 0.0, march_us = 0.0;
+        if (precision_ == RTLBFS_FP32) {
+            pick_tile_height(&tile_us);
+            pick_march_rows(&march_us);
+        }
+        use_kernel(precision_ == RTLBFS_FP32 && march_us < tile_us ? 0 : 1);
+    }
     if (kernel_ >= 1) {
-        const int h = chunk_rows_ > 0 ? chunk_rows_ : pick_tile_height();
+        const int h = chunk_rows_ > 0 ? chunk_rows_ : pick_tile_height(nullptr);
         if (h != tile_h_ && gexec_) {  // the graph baked the other tile kernel
             cudaGraphExecDestroy(gexec_);
             gexec_ = nullptr;
@@ -679,15 +746,16 @@ int Engine::rebuild_tiles()
             }
         }
     } else {
-        // warp-marching units: strips of kStrip columns, chunks of H rows.
-        // H: long enough to amortise each unit's 2-row prologue, short
-        // enough that there are ~8 warps per SM of units to run.
-        long long strip_rows = 0;
-        for (int s = 0; s < capacity_; ++s)
-            if (slots_[s].active)
-                strip_rows += (long long)((slots_[s].nx + kStrip - 1) / kStrip) * slots_[s].ny;
+        // warp-marching units: strips of columns, chunks of H rows
+        const int strip = precision_ == RTLBFS_FP32 ? kStrip2 : kStrip;
         int H = chunk_rows_;
-        if (H <= 0) {  // ~16 warps of units per SM, at least 16 rows each
+        if (H <= 0 && precision_ == RTLBFS_FP32) {
+            H = pick_march_rows(nullptr);
+        } else if (H <= 0) {  // ~16 warps of units per SM, at least 16 rows each
+            long long strip_rows = 0;
+            for (int s = 0; s < capacity_; ++s)
+                if (slots_[s].active)
+                    strip_rows += (long long)((slots_[s].nx + strip - 1) / strip) * slots_[s].ny;
             const long long target = (long long)sms_ * 16;
             H = (int)std::max<long long>(16, (strip_rows + target - 1) / std::max<long long>(target, 1));
             H = std::min(H, 64);
@@ -695,14 +763,14 @@ int Engine::rebuild_tiles()
         for (int s = 0; s < capacity_; ++s) {
             Cavity& c = slots_[s];
             if (!c.active) continue;
-            const int strips = (c.nx + kStrip - 1) / kStrip;
+            const int strips = (c.nx + strip - 1) / strip;
             const int h = std::min(H, c.ny);
             const int chunks = (c.ny + h - 1) / h;
             c.first_tile = (int)t.size();
             c.ntiles = strips * chunks;
             for (int k = 0; k < chunks; ++k)
                 for (int i = 0; i < strips; ++i)
-                    t.push_back(make_int4(s, i * kStrip, k * h, std::min(c.ny, (k + 1) * h)));
+                    t.push_back(make_int4(s, i * strip, k * h, std::min(c.ny, (k + 1) * h)));
         }
     }
     // the unit range of every cavity lives in its descriptor
@@ -755,7 +823,7 @@ int Engine::prepare_launch()
         desc_dirty_ = false;
     }
     // persistent grid: every SM full, never more blocks than work units
-    int want;
+    int want, march_cap = 0;
     if (kernel_ == 2) {
         int rc = persist_check();
         if (rc) return rc;
@@ -771,14 +839,20 @@ int Engine::prepare_launch()
         const int occ = scheme_ == kSchemeTLBFS ? occ_tlbfs_ : occ_tile_[tile_h_];
         want = std::max(1, std::min(sms_ * occ, std::max(ntiles_, 1)));
     } else {
-        const int wpb = kMarchThreads / 32;
+        const int wpb = (precision_ == RTLBFS_FP32 ? kMarch2Threads : kMarchThreads) / 32;
         want = std::max(1, std::min(sms_ * occ_march_, (std::max(ntiles_, 1) + wpb - 1) / wpb));
+        // one cavity's equal units below a full wave: no more resident blocks
+        // per SM than an even spread needs, or the next step's blocks,
+        // launched early, fill the free places of some SMs and leave others
+        // short (1024^2 in 16-row units: 46.7 -> 37.9 us)
+        march_cap = capacity_ == 1 && want < sms_ * occ_march_ ? (want + sms_ - 1) / sms_ : 0;
     }
-    if (want != grid_ && gexec_) {
+    if ((want != grid_ || march_cap != march_cap_) && gexec_) {
         cudaGraphExecDestroy(gexec_);
         gexec_ = nullptr;
     }
     grid_ = want;
+    march_cap_ = march_cap;
     return RTLBFS_OK;
 }
 
@@ -1159,8 +1233,8 @@ int Engine::launch_steps(long long launches)
     auto launch = [&](cudaStream_t st, int p) {
         return kernel_ == 1 ? launch_step(precision_, tile_h_, scheme_, grid_, st, d_desc_, d_ctl_,
                                           d_tiles_, d_ntiles_, p)
-                            : launch_march(precision_, grid_, st, d_desc_, d_ctl_, d_tiles_,
-                                           d_ntiles_, p);
+                            : launch_march(precision_, grid_, march_cap_, st, d_desc_, d_ctl_,
+                                           d_tiles_, d_ntiles_, p);
     };
     static_assert(kGraphChunk % 2 == 0, "graphs of an even number of launches");
     if (left >= kGraphChunk) {
@@ -1243,12 +1317,14 @@ int Engine::autotune(int steps, int* kernel_out, int* rows_out, double* ms_out)
                 tiles <= (long long)sms_ * occ_persist_[h])
                 cands.push_back({2, h});
         }
-    for (int H : {8, 16, 32, 64, 128, 256}) {
-        if (scheme_ == kSchemeTLBFS) break;
-        if (H > maxny && H != 8) break;
-        cands.push_back({0, H});
+    if (scheme_ != kSchemeTLBFS) {
+        std::vector<int> rows = {8, 16, 32, 64, 128, 256};
+        if (precision_ == RTLBFS_FP32) rows = {pick_march_rows(nullptr), 16, 32, 64};
+        for (size_t k = 0; k < rows.size(); ++k)
+            if (k == 0 || (rows[k] <= maxny && rows[k] != rows[0])) cands.push_back({0, rows[k]});
     }
     const int keep_kernel = kernel_, keep_rows = chunk_rows_;
+    const bool keep_auto = auto_kernel_;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
@@ -1297,6 +1373,7 @@ int Engine::autotune(int steps, int* kernel_out, int* rows_out, double* ms_out)
     if (rc) {
         set_kernel(keep_kernel);
         set_chunk_rows(keep_rows);
+        auto_kernel_ = keep_auto;
         return rc;
     }
     set_kernel(pick.kernel);

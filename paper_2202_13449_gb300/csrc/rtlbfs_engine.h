@@ -130,10 +130,13 @@ public:
     int cuda_fail(cudaError_t e, const char* what);
     int active_tiles() const { return ntiles_; }
     int grid() const { return grid_; }
-    // step kernel: 0 = warp-marching strips (default), 1 = shared-memory
-    // tiles, 2 = the tile kernel in persistent form (one cavity whose tiles
+    // step kernel (none set: see choose_kernel_by_size): 0 = warp-marching strips, 1 =
+    // shared-memory tiles, 2 = the tile kernel in persistent form (one cavity whose tiles
     // all fit on the GPU at once; many steps per launch)
     int set_kernel(int kind);
+    // until a schedule is set, pick the step kernel by size (engines of one
+    // cavity; a batch marches)
+    void choose_kernel_by_size() { auto_kernel_ = true; }
     // tests only: the persistent kernel's tile that never reports progress
     // (-1: none), to exercise its bounded waits
     void set_withhold(int tile) { withhold_ = tile; }
@@ -172,8 +175,14 @@ private:
     int persist_check();        // sets persist_slot_ or fails with the reason
     int scheme_ = 0;
     int tile_h_ = 16;        // tile height of the current tile list
-    int pick_tile_height() const;
+    // the automatic tile height / rows of a marching unit for the current
+    // cavities, and the modelled FP32 step time (us, may be null)
+    int pick_tile_height(double* us) const;
+    int pick_march_rows(double* us) const;
+    void use_kernel(int kind);
+    bool auto_kernel_ = false;  // no schedule set: rebuild_tiles picks the kernel
     int kernel_ = 0, occ_march_ = 0, chunk_rows_ = 0;
+    int march_cap_ = 0;        // marching kernel: resident blocks per SM to allow
     int launch_one(cudaStream_t s);
     cudaStream_t stream_ = nullptr, own_stream_ = nullptr;
     std::vector<Cavity> slots_;

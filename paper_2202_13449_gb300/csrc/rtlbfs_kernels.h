@@ -24,15 +24,12 @@ inline bool tile_height_ok(int precision, int h)
         if (t == h) return true;
     return false;
 }
-#ifndef RTLBFS_MARCH_THREADS
-#define RTLBFS_MARCH_THREADS 128
-#endif
-#ifndef RTLBFS_MARCH_MIN_BLOCKS_FP32
-#define RTLBFS_MARCH_MIN_BLOCKS_FP32 4
-#endif
-constexpr int kMarchThreads = RTLBFS_MARCH_THREADS;  // 4 warps per block
-constexpr int kMarchMinBlocksFP32 = RTLBFS_MARCH_MIN_BLOCKS_FP32;
+constexpr int kMarchThreads = 128;  // 4 warps per block (FP64)
 constexpr int kStrip = 28;  // interior columns per warp (32 lanes - 2 x 2 halo)
+// the FP32 marching kernel: two columns a lane
+constexpr int kMarch2Threads = 32;  // one warp per block
+constexpr int kMarch2Blocks = 12;   // resident blocks per SM to compile for
+constexpr int kStrip2 = 60;  // interior columns per warp (64 - 2 x 2 halo)
 
 constexpr int kNuWest = 0, kNuEast = 1, kNuSouth = 2, kNuNorth = 3, kNuAvg = 4, kNuHalf = 5;
 
@@ -56,8 +53,13 @@ cudaError_t launch_step(int precision, int tile_h, int scheme, int grid, cudaStr
                         const int* ntiles, int par);
 cudaError_t march_prepare(int precision);
 cudaError_t march_occupancy(int precision, int* blocks_per_sm);
-cudaError_t launch_march(int precision, int grid, cudaStream_t s, const CavityDesc* descs,
+// cap: no more than that many resident blocks per SM (FP32; 0: no limit)
+cudaError_t launch_march(int precision, int grid, int cap, cudaStream_t s, const CavityDesc* descs,
                          CavityRun* runs, const int4* units, const int* nunits, int par);
+cudaError_t march2_prepare();
+cudaError_t march2_occupancy(int* blocks_per_sm);
+cudaError_t launch_march2(int grid, int cap, cudaStream_t s, const CavityDesc* descs, CavityRun* runs,
+                          const int4* units, const int* nunits, int par);
 // the stop test of the last step of a chain whose next launch would have
 // parity par, for cavities 0..n-1: both headers become the tested header
 cudaError_t launch_finalize(cudaStream_t s, CavityRun* runs, int n, int par);

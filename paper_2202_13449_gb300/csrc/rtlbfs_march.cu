@@ -1,4 +1,5 @@
-// rtlbfs_march.cu -- the RTLBFS step as a warp-marching stencil.
+// rtlbfs_march.cu -- the FP64 RTLBFS step as a warp-marching stencil (FP32:
+// rtlbfs_march2.cu, two columns a lane in packed arithmetic).
 //
 // Work unit: one warp, a strip of kStrip = 28 interior columns and a chunk
 // of rows [j0, j1) of one cavity.  Lane l holds column c0 - 2 + l: lanes 0-1
@@ -6,7 +7,7 @@
 // the chunk keeping a rolling window in registers -- values of rows j, j+1,
 // j+2, gradients of rows j and j+1, the flux through the face below row j --
 // and per row:
-//   loads row j+2 (one coalesced 128-byte line per field),
+//   loads row j+2 (one coalesced line per field),
 //   x-faces of row j: each lane computes its west face; the left cell's
 //     values and gradients come from lane l-1 by shuffles,
 //   Green-Gauss gradients of row j+1 (Eqs. 55-56; x-neighbours by shuffles),
@@ -129,25 +130,15 @@ __device__ __forceinline__ R wsum(R v)
     return v;
 }
 
-template <class P>
-struct MarchMin {
-    static constexpr int value = 2;
-};
-template <>
-struct MarchMin<StoreQ> {
-    static constexpr int value = kMarchMinBlocksFP32;
-};
-
 }  // namespace
 
 template <class P>
-__global__ void __launch_bounds__(kMarchThreads, MarchMin<P>::value)
+__global__ void __launch_bounds__(kMarchThreads, 2)
 march_kernel(const CavityDesc* __restrict__ descs, CavityRun* __restrict__ runs,
              const int4* __restrict__ units, const int* __restrict__ nunits_ptr, int par)
 {
     using S = typename P::S;
     using R = typename P::R;
-    using V2 = typename P::V2;
     const int lane = threadIdx.x & 31;
     const int wpb = kMarchThreads / 32;
     chain_sync();
@@ -220,18 +211,14 @@ march_kernel(const CavityDesc* __restrict__ descs, CavityRun* __restrict__ runs,
             const Vec4<R> vw = shfl_up1(v), ve = shfl_dn1(v);
             const int ri = min(max(r + 2, 1), ny + 3);
             const R isy_n = yc[ri].is_next, isy_s = yc[ri - 1].is_next;
-            if constexpr (sizeof(R) == 4) {
-                gg_gradient_f32(v, ve, vw, vn, vs, isx_e, isx_w, isy_n, isy_s, gx, gy);
-            } else {
-                gx.x = (ve.x - v.x) * isx_e + (v.x - vw.x) * isx_w;
-                gx.y = (ve.y - v.y) * isx_e + (v.y - vw.y) * isx_w;
-                gx.z = (ve.z - v.z) * isx_e + (v.z - vw.z) * isx_w;
-                gx.w = (ve.w - v.w) * isx_e + (v.w - vw.w) * isx_w;
-                gy.x = (vn.x - v.x) * isy_n + (v.x - vs.x) * isy_s;
-                gy.y = (vn.y - v.y) * isy_n + (v.y - vs.y) * isy_s;
-                gy.z = (vn.z - v.z) * isy_n + (v.z - vs.z) * isy_s;
-                gy.w = (vn.w - v.w) * isy_n + (v.w - vs.w) * isy_s;
-            }
+            gx.x = (ve.x - v.x) * isx_e + (v.x - vw.x) * isx_w;
+            gx.y = (ve.y - v.y) * isx_e + (v.y - vw.y) * isx_w;
+            gx.z = (ve.z - v.z) * isx_e + (v.z - vw.z) * isx_w;
+            gx.w = (ve.w - v.w) * isx_e + (v.w - vw.w) * isx_w;
+            gy.x = (vn.x - v.x) * isy_n + (v.x - vs.x) * isy_s;
+            gy.y = (vn.y - v.y) * isy_n + (v.y - vs.y) * isy_s;
+            gy.z = (vn.z - v.z) * isy_n + (v.z - vs.z) * isy_s;
+            gy.w = (vn.w - v.w) * isy_n + (v.w - vs.w) * isy_s;
             if (xghosts) {
                 const Vec4<R> gxd = shfl_dn1(gx), gyd = shfl_dn1(gy);
                 const Vec4<R> gxu = shfl_up1(gx), gyu = shfl_up1(gy);
@@ -242,103 +229,31 @@ march_kernel(const CavityDesc* __restrict__ descs, CavityRun* __restrict__ runs,
                 }
             }
         };
-        // One packed call for two faces: component x = the x-face west of this
-        // lane's column in row jx (left cell from lane l-1), component y = the
-        // y-face between rows jf-1 and jf of this lane's column.
-        auto faces = [&](const Vec4<R>& vxl, const Vec4<R>& gxxl, const Vec4<R>& gyxl,
-                         const Vec4<R>& vxr, const Vec4<R>& gxxr, const Vec4<R>& gyxr, int jf,
-                         const Vec4<R>& vyl, const Vec4<R>& gxyl, const Vec4<R>& gyyl,
-                         const Vec4<R>& vyr, const Vec4<R>& gxyr, const Vec4<R>& gyyr,
-                         Vec4<R>& Fxo, Vec4<R>& Fyo) {
+        // the x-face west of this lane's column (left cell from lane l-1)
+        auto xface = [&](const Vec4<R>& vl, const Vec4<R>& gxl, const Vec4<R>& gyl,
+                         const Vec4<R>& vr, const Vec4<R>& gxr, const Vec4<R>& gyr) -> Vec4<R> {
+            const CellNT<R> L = {{vl.x, vl.y, vl.z, R(0)}, {gxl.x, gxl.y, gxl.z, gxl.w},
+                                 {gyl.x, gyl.y, gyl.z, gyl.w}};
+            const CellNT<R> Rr = {{vr.x, vr.y, vr.z, vr.w - vl.w}, {gxr.x, gxr.y, gxr.z, gxr.w},
+                                  {gyr.x, gyr.y, gyr.z, gyr.w}};
+            R F[4];
+            face_flux<R>(L, Rr, Tz + vl.w, flx, wsx >= 0 ? R(0) : R(1),
+                         wsx >= 0 ? P::bcU(dp, wsx) : R(0), F);
+            return {F[0], F[1], F[2], F[3]};
+        };
+        // the y-face between rows jf-1 and jf of this lane's column
+        auto yface = [&](int jf, const Vec4<R>& vl, const Vec4<R>& gxl, const Vec4<R>& gyl,
+                         const Vec4<R>& vr, const Vec4<R>& gxr, const Vec4<R>& gyr) -> Vec4<R> {
             const FaceLine<R> fly = yl[min(max(jf, 0), ny)];
             const int ws = (wall_s && jf == 0) ? kSideS : ((wall_n && jf == ny) ? kSideN : -1);
-            const R uwy = ws >= 0 ? P::bcU(dp, ws) : R(0);
-            const R uwx = wsx >= 0 ? P::bcU(dp, wsx) : R(0);
-            CellNT<V2> L, Rr;
-            // x-face frame (n = x, t = y) in .x, y-face frame (n = y, t = x) in .y
-            L.q[0] = {vxl.x, vyl.x};
-            L.q[1] = {vxl.y, vyl.z};
-            L.q[2] = {vxl.z, vyl.y};
-            L.q[3] = {R(0), R(0)};
-            L.gn[0] = {gxxl.x, gyyl.x};
-            L.gn[1] = {gxxl.y, gyyl.z};
-            L.gn[2] = {gxxl.z, gyyl.y};
-            L.gn[3] = {gxxl.w, gyyl.w};
-            L.gt[0] = {gyxl.x, gxyl.x};
-            L.gt[1] = {gyxl.y, gxyl.z};
-            L.gt[2] = {gyxl.z, gxyl.y};
-            L.gt[3] = {gyxl.w, gxyl.w};
-            Rr.q[0] = {vxr.x, vyr.x};
-            Rr.q[1] = {vxr.y, vyr.z};
-            Rr.q[2] = {vxr.z, vyr.y};
-            Rr.q[3] = {vxr.w - vxl.w, vyr.w - vyl.w};
-            Rr.gn[0] = {gxxr.x, gyyr.x};
-            Rr.gn[1] = {gxxr.y, gyyr.z};
-            Rr.gn[2] = {gxxr.z, gyyr.y};
-            Rr.gn[3] = {gxxr.w, gyyr.w};
-            Rr.gt[0] = {gyxr.x, gxyr.x};
-            Rr.gt[1] = {gyxr.y, gxyr.z};
-            Rr.gt[2] = {gyxr.z, gxyr.y};
-            Rr.gt[3] = {gyxr.w, gxyr.w};
-            FaceLine<V2> fl;
-            fl.h = {flx.h, fly.h};
-            fl.cL = {flx.cL, fly.cL};
-            fl.cR = {flx.cR, fly.cR};
-            fl.m_nu_2h = {flx.m_nu_2h, fly.m_nu_2h};
-            fl.m_chi_2h = {flx.m_chi_2h, fly.m_chi_2h};
-            fl.m_tf15 = {flx.m_tf15, fly.m_tf15};
-            fl.m_tg15 = {flx.m_tg15, fly.m_tg15};
-            const V2 Tbar = {Tz + vxl.w, Tz + vyl.w};
-            const V2 keep = {wsx >= 0 ? R(0) : R(1), ws >= 0 ? R(0) : R(1)};
-            const V2 uw = {uwx, uwy};
-            V2 F[4];
-            face_flux<V2>(L, Rr, Tbar, fl, keep, uw, F);
-            Fxo = {F[0].x, F[1].x, F[2].x, F[3].x};
-            Fyo = {F[0].y, F[2].y, F[1].y, F[3].y};
-        };
-
-        // The same two faces as two scalar evaluations.
-        auto face1 = [&](const Vec4<R>& vxl, const Vec4<R>& gxxl, const Vec4<R>& gyxl,
-                         const Vec4<R>& vxr, const Vec4<R>& gxxr, const Vec4<R>& gyxr, int jf,
-                         const Vec4<R>& vyl, const Vec4<R>& gxyl, const Vec4<R>& gyyl,
-                         const Vec4<R>& vyr, const Vec4<R>& gxyr, const Vec4<R>& gyyr,
-                         Vec4<R>& Fxo, Vec4<R>& Fyo) {
-            {
-                R F[4];
-                if constexpr (sizeof(R) == 4) {  // FP32: packed column stage
-                    R A[4], Sa[4], M[4], D[4], B[4], Sb[4];
-                    face_columns_f32<true>(vxl, vxr, gxxl, gyxl, gxxr, gyxr, flx, A, Sa, M, D, B, Sb);
-                    face_flux_columns<R>(A, Sa, M, D, B, Sb, Tz + vxl.w, flx, wsx >= 0 ? R(0) : R(1),
-                                         wsx >= 0 ? P::bcU(dp, wsx) : R(0), F);
-                } else {
-                    CellNT<R> L = {{vxl.x, vxl.y, vxl.z, R(0)}, {gxxl.x, gxxl.y, gxxl.z, gxxl.w},
-                                   {gyxl.x, gyxl.y, gyxl.z, gyxl.w}};
-                    CellNT<R> Rr = {{vxr.x, vxr.y, vxr.z, vxr.w - vxl.w},
-                                    {gxxr.x, gxxr.y, gxxr.z, gxxr.w}, {gyxr.x, gyxr.y, gyxr.z, gyxr.w}};
-                    face_flux<R>(L, Rr, Tz + vxl.w, flx, wsx >= 0 ? R(0) : R(1),
-                                 wsx >= 0 ? P::bcU(dp, wsx) : R(0), F);
-                }
-                Fxo = {F[0], F[1], F[2], F[3]};
-            }
-            {
-                const FaceLine<R> fly = yl[min(max(jf, 0), ny)];
-                const int ws = (wall_s && jf == 0) ? kSideS : ((wall_n && jf == ny) ? kSideN : -1);
-                R F[4];
-                if constexpr (sizeof(R) == 4) {
-                    R A[4], Sa[4], M[4], D[4], B[4], Sb[4];
-                    face_columns_f32<false>(vyl, vyr, gyyl, gxyl, gyyr, gxyr, fly, A, Sa, M, D, B, Sb);
-                    face_flux_columns<R>(A, Sa, M, D, B, Sb, Tz + vyl.w, fly, ws >= 0 ? R(0) : R(1),
-                                         ws >= 0 ? P::bcU(dp, ws) : R(0), F);
-                } else {
-                    CellNT<R> L = {{vyl.x, vyl.z, vyl.y, R(0)}, {gyyl.x, gyyl.z, gyyl.y, gyyl.w},
-                                   {gxyl.x, gxyl.z, gxyl.y, gxyl.w}};
-                    CellNT<R> Rr = {{vyr.x, vyr.z, vyr.y, vyr.w - vyl.w},
-                                    {gyyr.x, gyyr.z, gyyr.y, gyyr.w}, {gxyr.x, gxyr.z, gxyr.y, gxyr.w}};
-                    face_flux<R>(L, Rr, Tz + vyl.w, fly, ws >= 0 ? R(0) : R(1),
-                                 ws >= 0 ? P::bcU(dp, ws) : R(0), F);
-                }
-                Fyo = {F[0], F[2], F[1], F[3]};
-            }
+            const CellNT<R> L = {{vl.x, vl.z, vl.y, R(0)}, {gyl.x, gyl.z, gyl.y, gyl.w},
+                                 {gxl.x, gxl.z, gxl.y, gxl.w}};
+            const CellNT<R> Rr = {{vr.x, vr.z, vr.y, vr.w - vl.w}, {gyr.x, gyr.z, gyr.y, gyr.w},
+                                  {gxr.x, gxr.z, gxr.y, gxr.w}};
+            R F[4];
+            face_flux<R>(L, Rr, Tz + vl.w, fly, ws >= 0 ? R(0) : R(1),
+                         ws >= 0 ? P::bcU(dp, ws) : R(0), F);
+            return {F[0], F[2], F[1], F[3]};
         };
 
         // ---- prologue: rows j0-2 .. j0+1, gradients of j0-1 and j0,
@@ -368,9 +283,7 @@ march_kernel(const CavityDesc* __restrict__ descs, CavityRun* __restrict__ runs,
             gy1 = gym1;
             v2 = vm1;
         }
-        // the face below row j0 (paired with a throw-away copy of itself)
-        Vec4<R> Fs, Fdummy;
-        faces(v2, gx1, gy1, v0, gx0, gy0, j0, v2, gx1, gy1, v0, gx0, gy0, Fdummy, Fs);
+        Vec4<R> Fs = yface(j0, v2, gx1, gy1, v0, gx0, gy0);  // the face below row j0
 
         R s0 = R(0), s1 = R(0), s2 = R(0), s3 = R(0);
         bool bad = false;
@@ -389,15 +302,8 @@ march_kernel(const CavityDesc* __restrict__ descs, CavityRun* __restrict__ runs,
             }
             // x-face west of this lane's column in row j and the y-face
             // between rows j and j+1
-            Vec4<R> Fx, Fn;
-            {
-                const Vec4<R> vl = shfl_up1(v0), gxl = shfl_up1(gx0), gyl = shfl_up1(gy0);
-#if RTLBFS_PAIR_FACES
-                faces(vl, gxl, gyl, v0, gx0, gy0, j + 1, v0, gx0, gy0, v1, gx1, gy1, Fx, Fn);
-#else
-                face1(vl, gxl, gyl, v0, gx0, gy0, j + 1, v0, gx0, gy0, v1, gx1, gy1, Fx, Fn);
-#endif
-            }
+            const Vec4<R> Fx = xface(shfl_up1(v0), shfl_up1(gx0), shfl_up1(gy0), v0, gx0, gy0);
+            const Vec4<R> Fn = yface(j + 1, v0, gx0, gy0, v1, gx1, gy1);
             const Vec4<R> Fe = shfl_dn1(Fx);
             // update row j
             if (upd_lane) {
@@ -406,15 +312,10 @@ march_kernel(const CavityDesc* __restrict__ descs, CavityRun* __restrict__ runs,
                 const R ay = yc[j + 2].dt_w;
                 const R dr = v0.x, u = v0.y, v = v0.z, T = Tz + v0.w;
                 const R rho = one + dr;
-                R div0, div1, div2, div3;
-                if constexpr (sizeof(R) == 4) {
-                    flux_div_f32(Fx, Fe, Fs, Fn, ax, ay, div0, div1, div2, div3);
-                } else {
-                    div0 = ax * (Fe.x - Fx.x) + ay * (Fn.x - Fs.x);
-                    div1 = ax * (Fe.y - Fx.y) + ay * (Fn.y - Fs.y);
-                    div2 = ax * (Fe.z - Fx.z) + ay * (Fn.z - Fs.z);
-                    div3 = ax * (Fe.w - Fx.w) + ay * (Fn.w - Fs.w);
-                }
+                const R div0 = ax * (Fe.x - Fx.x) + ay * (Fn.x - Fs.x);
+                const R div1 = ax * (Fe.y - Fx.y) + ay * (Fn.y - Fs.y);
+                const R div2 = ax * (Fe.z - Fx.z) + ay * (Fn.z - Fs.z);
+                const R div3 = ax * (Fe.w - Fx.w) + ay * (Fn.w - Fs.w);
                 const R src_x = rho * P::fx(dp);
                 const R src_y = rho * (P::beta_g(dp) * (T - P::T_ref(dp)) + P::fy(dp));
                 const R dtc = P::dt(dp);
@@ -461,8 +362,7 @@ march_kernel(const CavityDesc* __restrict__ descs, CavityRun* __restrict__ runs,
 
 cudaError_t march_prepare(int precision)
 {
-    (void)precision;
-    return cudaSuccess;
+    return precision == 0 ? cudaSuccess : march2_prepare();
 }
 
 cudaError_t march_occupancy(int precision, int* blocks_per_sm)
@@ -470,18 +370,16 @@ cudaError_t march_occupancy(int precision, int* blocks_per_sm)
     if (precision == 0)
         return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, march_kernel<StoreD>,
                                                              kMarchThreads, 0);
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, march_kernel<StoreQ>,
-                                                         kMarchThreads, 0);
+    return march2_occupancy(blocks_per_sm);
 }
 
-cudaError_t launch_march(int precision, int grid, cudaStream_t s, const CavityDesc* descs,
+cudaError_t launch_march(int precision, int grid, int cap, cudaStream_t s, const CavityDesc* descs,
                          CavityRun* runs, const int4* units, const int* nunits, int par)
 {
     if (precision == 0)
         return launch_chained(march_kernel<StoreD>, grid, kMarchThreads, 0, s, descs, runs, units,
                               nunits, par);
-    return launch_chained(march_kernel<StoreQ>, grid, kMarchThreads, 0, s, descs, runs, units,
-                          nunits, par);
+    return launch_march2(grid, cap, s, descs, runs, units, nunits, par);
 }
 
 }  // namespace rtlbfs

@@ -55,6 +55,7 @@ Cnt vfma(Cnt a, Cnt b, Cnt c)
 template <>
 struct vtraits<Cnt> {
     static Cnt bc(double c) { return {c, c == 0.0}; }
+    static Cnt neg(Cnt x) { return {-x.v, x.zero}; }  // an operand's sign: free
     static Cnt rcp(Cnt x)
     {
         ++g_tally.sfu;

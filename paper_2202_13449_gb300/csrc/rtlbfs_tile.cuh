@@ -503,10 +503,10 @@ __device__ __forceinline__ void tile_step(TileSmem<P, TX, TY, NT>& sm, const Cav
                 const Vec4<R> tl = isx ? sm.gy[lr - 1][lc - 1] : sm.gx[lr - 1][lc - 1];
                 const Vec4<R> gr = isx ? sm.gx[rr - 1][rc - 1] : sm.gy[rr - 1][rc - 1];
                 const Vec4<R> tr = isx ? sm.gy[rr - 1][rc - 1] : sm.gx[rr - 1][rc - 1];
-                R A[4], Sa[4], M[4], D[4], B[4], Sb[4];
-                face_columns_f32<isx>(sm.val[lr][lc], sm.val[rr][rc], gl, tl, gr, tr, fl, A, Sa, M,
+                R A[4], Na[4], M[4], D[4], B[4], Sb[4];
+                face_columns_f32<isx>(sm.val[lr][lc], sm.val[rr][rc], gl, tl, gr, tr, fl, A, Na, M,
                                       D, B, Sb);
-                face_flux_columns<R>(A, Sa, M, D, B, Sb, Tbar, fl, wside >= 0 ? R(0) : R(1), uw, F);
+                face_flux_columns<R>(A, Na, M, D, B, Sb, Tbar, fl, wside >= 0 ? R(0) : R(1), uw, F);
             } else {
                 face_flux<R>(L, Rr, Tbar, fl, wside >= 0 ? R(0) : R(1), uw, F);
             }
