@@ -250,8 +250,8 @@ int rtlbfs_set_scheme(rtlbfs_t h, int scheme);
  * kernel 0 = warp-marching strips (each warp walks a strip of 60 columns, 28
  * in FP64, up a chunk of chunk_rows rows, rolling its stencil window in
  * registers; chunk_rows 0 = chosen from the GPU size), kernel 1 = shared-memory tiles
- * of 32 columns by chunk_rows rows (16, 14, 12, 10, 8, 4 or 2 in FP32; 16,
- * 8, 4 or 2 in FP64; 0 = the height whose tile count fills the SMs most
+ * of 32 columns (FP64, 2 rows: 16) by chunk_rows rows (16, 14, 12, 10, 8, 4 or
+ * 2 in FP32; 16, 8, 4 or 2 in FP64; 0 = the height whose tile count fills the SMs most
  * evenly), kernel 2 = the same tiles in one persistent cooperative launch
  * per chunk of steps, each tile waiting only for the eight around it (the
  * RTLBFS stage, every tile resident at once and at least 2 cells wide; the

@@ -152,7 +152,11 @@ int Engine::init()
     CK(persist_prepare(precision_));
     for (int h : kTileHeights) {
         if (!tile_height_ok(precision_, h)) continue;
-        CK(persist_occupancy(precision_, h, &occ_persist_[h]));
+        // the smaller of the two widths a height may run at
+        int wide = 0;
+        CK(persist_occupancy(precision_, kTileX, h, &wide));
+        CK(persist_occupancy(precision_, tile_width(precision_, h), h, &occ_persist_[h]));
+        occ_persist_[h] = std::min(occ_persist_[h], wide);
     }
     CK(march_prepare(precision_));
     CK(march_occupancy(precision_, &occ_march_));
@@ -532,7 +536,7 @@ int Engine::upload_lines(int slot)
         d.bcT[s] = c.bcT[s] / Tu;
         d.bcU[s] = c.bcU[s];
     }
-    d.tiles_x = (c.nx + kTileX - 1) / kTileX;
+    d.tiles_x = (c.nx + tile_w_ - 1) / tile_w_;
     d.tiles_y = (c.ny + tile_h_ - 1) / tile_h_;
     d.scheme = scheme_;
     d.ntiles = c.ntiles;  // work units of this cavity in the current list
@@ -634,9 +638,10 @@ int Engine::set_chunk_rows(int rows)
 // the residual), in face-equivalents: 65 h + 32 + 0.25 * 34 (h + 2) + 300.
 // FP32 leaves out heights below 8: one or two warps a block pass through a
 // tile's phases too slowly even when every tile has an SM of its own (64^2:
-// 10.0 us per step at h = 2, 7.0 at 4, 6.6 at 8, 6.7 at 14).  FP64 counts a
-// 16-row tile 1.17 times: one such block fills an SM's registers and its
-// phases overlap with nothing (400^2: 228 us at h = 16, 194 at 8).
+// 10.0 us per step at h = 2, 7.0 at 4, 6.6 at 8, 6.7 at 14).  FP64 is bound
+// by its narrow units, for which every warp instruction counts the same
+// however few lanes it serves: the cost is a tile's FP64 warp instructions
+// (rounds of faces 175, of gradients 32, of updates 170).
 int Engine::pick_tile_height(double* us) const
 {
     if (scheme_ == kSchemeTLBFS) return kTileYDefault;
@@ -646,14 +651,16 @@ int Engine::pick_tile_height(double* us) const
     for (int h : kTileHeights) {
         if (!tile_height_ok(precision_, h)) continue;
         if (precision_ == RTLBFS_FP32 && h < 8) continue;
+        const int w = tile_width(precision_, h);
         long long tiles = 0;
         for (int s = 0; s < capacity_; ++s)
             if (slots_[s].active)
-                tiles += (long long)((slots_[s].nx + kTileX - 1) / kTileX) *
-                         ((slots_[s].ny + h - 1) / h);
+                tiles += (long long)((slots_[s].nx + w - 1) / w) * ((slots_[s].ny + h - 1) / h);
         const long long deep = (tiles + sms_ - 1) / std::max(sms_, 1);
-        double cost = (double)deep * (65.0 * h + 32.0 + 0.25 * 34.0 * (h + 2) + 300.0);
-        if (precision_ == RTLBFS_FP64 && h == 16) cost *= 1.17;
+        const double tile_cost =
+            precision_ == RTLBFS_FP64 ? (h == 2 ? 900.0 : h == 4 ? 2654.0 : h == 8 ? 4862.0 : 9310.0)
+                                      : 65.0 * h + 32.0 + 0.25 * 34.0 * (h + 2) + 300.0;
+        const double cost = (double)deep * tile_cost;
         if (cost < best * (1.0 - 1e-9)) {
             best = cost;
             best_h = h;
@@ -725,14 +732,21 @@ int Engine::rebuild_tiles()
             gexec_ = nullptr;
         }
         tile_h_ = h;
+        // the persistent kernel takes no tile of one column: 32 columns where
+        // the narrower tile would leave one
+        tile_w_ = tile_width(precision_, h);
+        if (kernel_ == 2)
+            for (int s = 0; s < capacity_; ++s)
+                if (slots_[s].active && slots_[s].nx % tile_w_ == 1) tile_w_ = kTileX;
         for (int s = 0; s < capacity_; ++s) {
             Cavity& c = slots_[s];
             if (!c.active) continue;
-            const int tx = (c.nx + kTileX - 1) / kTileX, ty = (c.ny + tile_h_ - 1) / tile_h_;
+            const int tw = tile_w_;
+            const int tx = (c.nx + tw - 1) / tw, ty = (c.ny + tile_h_ - 1) / tile_h_;
             c.first_tile = (int)t.size();
             c.ntiles = tx * ty;
             for (int j = 0; j < ty; ++j)
-                for (int i = 0; i < tx; ++i) t.push_back(make_int4(s, i * kTileX, j * tile_h_, 0));
+                for (int i = 0; i < tx; ++i) t.push_back(make_int4(s, i * tw, j * tile_h_, 0));
             // Tiles whose halo reaches past the mesh edge take the ghost-resolution
             // path and run longer: spaced evenly through the cavity's part of the
             // list, they are spread over the SMs instead of several landing on one.
@@ -741,7 +755,7 @@ int Engine::rebuild_tiles()
             if (kernel_ == 1) {
                 const int nx = c.nx, ny = c.ny, th = tile_h_;
                 spread_units(t, (std::size_t)c.first_tile, [=](const int4& u) {
-                    return !(u.y >= 2 && u.z >= 2 && u.y + kTileX + 2 <= nx && u.z + th + 2 <= ny);
+                    return !(u.y >= 2 && u.z >= 2 && u.y + tw + 2 <= nx && u.z + th + 2 <= ny);
                 });
             }
         }
@@ -780,7 +794,7 @@ int Engine::rebuild_tiles()
         CavityDesc& d = h_desc_[s];
         d.ntiles = c.ntiles;
         d.tile_begin = c.first_tile;
-        d.tiles_x = (c.nx + kTileX - 1) / kTileX;
+        d.tiles_x = (c.nx + tile_w_ - 1) / tile_w_;
         d.tiles_y = (c.ny + tile_h_ - 1) / tile_h_;
     }
     desc_dirty_ = true;
@@ -1192,7 +1206,7 @@ int Engine::persist_check()
     const Cavity& c = slots_[slot];
     if (c.halo_rows)
         return fail(RTLBFS_ERR_ARG, "the persistent kernel takes whole meshes, not row strips");
-    if ((c.nx % kTileX) == 1 || (c.ny % tile_h_) == 1)
+    if ((c.nx % tile_w_) == 1 || (c.ny % tile_h_) == 1)
         return fail(RTLBFS_ERR_ARG, "the persistent kernel needs tiles at least 2 cells wide");
     if ((long long)ntiles_ > (long long)sms_ * occ_persist_[tile_h_])
         return fail(RTLBFS_ERR_ARG, "the mesh has more tiles than fit on the GPU at once");
@@ -1213,7 +1227,7 @@ int Engine::launch_steps(long long launches)
             const int n = (int)std::min<long long>(left, kPersistChunk);
             CK(cudaMemsetAsync(d_tstep_, 0, sizeof(int) * ntiles_, stream_));
             CK(cudaMemsetAsync(d_pctl_, 0, sizeof(PersistCtl), stream_));
-            CK(launch_persist(precision_, tile_h_, ntiles_, stream_, &d_desc_[persist_slot_],
+            CK(launch_persist(precision_, tile_w_, tile_h_, ntiles_, stream_, &d_desc_[persist_slot_],
                               &d_ctl_[persist_slot_].h[0], d_tiles_ + c.first_tile, d_tstep_, d_pctl_,
                               n, withhold_));
             g_launches++;
@@ -1311,8 +1325,8 @@ int Engine::autotune(int steps, int* kernel_out, int* rows_out, double* ms_out)
         for (int h : kTileHeights) {
             if (!tile_height_ok(precision_, h)) continue;
             const Cavity& c = slots_[aslot];
-            const long long tiles =
-                (long long)((c.nx + kTileX - 1) / kTileX) * ((c.ny + h - 1) / h);
+            const int w = c.nx % tile_width(precision_, h) == 1 ? kTileX : tile_width(precision_, h);
+            const long long tiles = (long long)((c.nx + w - 1) / w) * ((c.ny + h - 1) / h);
             if ((c.nx % kTileX) != 1 && (c.ny % h) != 1 &&
                 tiles <= (long long)sms_ * occ_persist_[h])
                 cands.push_back({2, h});

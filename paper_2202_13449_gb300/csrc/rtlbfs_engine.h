@@ -174,7 +174,7 @@ private:
     int persist_slot_ = -1;     // the one active cavity, once eligible
     int persist_check();        // sets persist_slot_ or fails with the reason
     int scheme_ = 0;
-    int tile_h_ = 16;        // tile height of the current tile list
+    int tile_h_ = 16, tile_w_ = kTileX;  // tile of the current tile list
     // the automatic tile height / rows of a marching unit for the current
     // cavities, and the modelled FP32 step time (us, may be null)
     int pick_tile_height(double* us) const;

@@ -8,15 +8,19 @@
 
 namespace rtlbfs {
 
-// Tiles of the shared-memory step kernel: kTileX = 32 columns by one of
-// the compiled heights below, 16 threads per tile row (two cells per thread
-// in the update).  The height is picked per cavity set so that the number of
+// Tiles of the shared-memory step kernel: kTileX = 32 columns (16 for the
+// 2-row FP64 tile, see tile_width) by one of the compiled heights below, 16
+// threads per tile row (two cells per thread in the update).  The height is picked per cavity set so that the number of
 // tiles fills the SMs evenly (a 512-row mesh in 16-row tiles leaves a third
 // of the SMs one tile short); the low heights spread small meshes over many
 // SMs, which matters most in FP64, where an SM does 2 FMAs per clock.
 constexpr int kTileX = 32;
 constexpr int kTileHeights[] = {16, 14, 12, 10, 8, 4, 2};
 constexpr int kTileYDefault = 16;
+// Columns of a tile.  The 2-row FP64 tile is 16 wide, 32 cells: the finest
+// spread of a small mesh over the SMs, whose narrow FP64 units bound the
+// step (tile_step_flat).  A 64^2 mesh has 128 such tiles, 64 of 32 columns.
+constexpr int tile_width(int precision, int h) { return precision == 0 && h == 2 ? 16 : kTileX; }
 inline bool tile_height_ok(int precision, int h)
 {
     if (precision == 0) return h == 16 || h == 8 || h == 4 || h == 2;
@@ -79,8 +83,9 @@ struct PersistCtl {
 // ntiles ints zeroed before the launch.  withhold >= 0 (tests only): that
 // tile never reports its progress, so the waits of its neighbours run out.
 cudaError_t persist_prepare(int precision);
-cudaError_t persist_occupancy(int precision, int tile_h, int* blocks_per_sm);
-cudaError_t launch_persist(int precision, int tile_h, int ntiles, cudaStream_t s,
+// tile_w: tile_width, or kTileX where that would leave a tile of one column
+cudaError_t persist_occupancy(int precision, int tile_w, int tile_h, int* blocks_per_sm);
+cudaError_t launch_persist(int precision, int tile_w, int tile_h, int ntiles, cudaStream_t s,
                            const CavityDesc* desc, CavityCtl* ctl, const int4* tiles, int* tstep,
                            PersistCtl* pc, int nsteps, int withhold);
 cudaError_t launch_nusselt(int precision, cudaStream_t s, const CavityDesc* descs,

@@ -149,9 +149,9 @@ persist_kernel(const CavityDesc* __restrict__ dp, CavityCtl* __restrict__ ctl,
         __syncthreads();
         if (sm.last != 1) break;  // uniform: stopped, or stalled
         const int rb = c0 ^ ((k - 1) & 1);  // buffer with the state after step k - 1
-        tile_step<P, TX, TY, NT, 0, true>(sm, &sm.desc, i0, j0,
-                                          static_cast<const Vec4<S>*>(dp->f[rb][0]),
-                                          static_cast<Vec4<S>*>(dp->f[rb ^ 1][0]), true);
+        run_tile<P, TX, TY, NT, 0, true>(sm, &sm.desc, i0, j0,
+                                         static_cast<const Vec4<S>*>(dp->f[rb][0]),
+                                         static_cast<Vec4<S>*>(dp->f[rb ^ 1][0]), true);
         __syncthreads();
         double a[4];
         if (tid < 32) tile_sums(sm, a);
@@ -189,11 +189,11 @@ persist_kernel(const CavityDesc* __restrict__ dp, CavityCtl* __restrict__ ctl,
     }
 }
 
-template <class P, int TY>
+template <class P, int TY, int TX = kTileX>
 struct PersistKernel {
-    static constexpr int NT = TileThreads<P, TY>::value;
-    static constexpr size_t smem = sizeof(TileSmem<P, kTileX, TY, NT>);
-    static constexpr auto fn = persist_kernel<P, kTileX, TY, NT>;
+    static constexpr int NT = TileThreads<P, TX, TY>::value;
+    static constexpr size_t smem = sizeof(TileSmem<P, TX, TY, NT>);
+    static constexpr auto fn = persist_kernel<P, TX, TY, NT>;
     static cudaError_t prepare()
     {
         cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -224,8 +224,13 @@ struct PersistKernel {
 };
 
 template <class Op>
-static cudaError_t with_persist_kernel(int precision, int tile_h, Op op)
+static cudaError_t with_persist_kernel(int precision, int tile_w, int tile_h, Op op)
 {
+    if (tile_w != kTileX) {
+        if (precision == 0 && tile_h == 2 && tile_w == tile_width(0, 2))
+            return op(PersistKernel<StoreD, 2, tile_width(0, 2)>());
+        return cudaErrorInvalidValue;
+    }
     if (precision == 0) {
         switch (tile_h) {
         case 16: return op(PersistKernel<StoreD, 16>());
@@ -251,23 +256,25 @@ cudaError_t persist_prepare(int precision)
 {
     for (int h : kTileHeights) {
         if (!tile_height_ok(precision, h)) continue;
-        cudaError_t e = with_persist_kernel(precision, h, [](auto k) { return k.prepare(); });
-        if (e != cudaSuccess) return e;
+        for (int w : {kTileX, tile_width(precision, h)}) {
+            cudaError_t e = with_persist_kernel(precision, w, h, [](auto k) { return k.prepare(); });
+            if (e != cudaSuccess) return e;
+        }
     }
     return cudaSuccess;
 }
 
-cudaError_t persist_occupancy(int precision, int tile_h, int* blocks_per_sm)
+cudaError_t persist_occupancy(int precision, int tile_w, int tile_h, int* blocks_per_sm)
 {
-    return with_persist_kernel(precision, tile_h,
+    return with_persist_kernel(precision, tile_w, tile_h,
                                [&](auto k) { return k.occupancy(blocks_per_sm); });
 }
 
-cudaError_t launch_persist(int precision, int tile_h, int ntiles, cudaStream_t s,
+cudaError_t launch_persist(int precision, int tile_w, int tile_h, int ntiles, cudaStream_t s,
                            const CavityDesc* desc, CavityCtl* ctl, const int4* tiles, int* tstep,
                            PersistCtl* pc, int nsteps, int withhold)
 {
-    return with_persist_kernel(precision, tile_h, [&](auto k) {
+    return with_persist_kernel(precision, tile_w, tile_h, [&](auto k) {
         return k.launch(ntiles, s, desc, ctl, tiles, tstep, pc, nsteps, withhold);
     });
 }

@@ -74,9 +74,9 @@ step_kernel(const CavityDesc* __restrict__ descs, CavityRun* __restrict__ runs,
         // their descriptor in place and load their lines beside the state
         const bool first = t == (int)blockIdx.x;
         const CavityDesc* dp = first ? &sm.desc : &descs[slot];
-        tile_step<P, TX, TY, NT, SCHEME, false>(sm, dp, i0, j0,
-                                                static_cast<const Vec4<S>*>(dp->f[cur][0]),
-                                                static_cast<Vec4<S>*>(dp->f[cur ^ 1][0]), first);
+        run_tile<P, TX, TY, NT, SCHEME, false>(sm, dp, i0, j0,
+                                               static_cast<const Vec4<S>*>(dp->f[cur][0]),
+                                               static_cast<Vec4<S>*>(dp->f[cur ^ 1][0]), first);
         __syncthreads();
         double a[4];
         if (tid < 32) tile_sums(sm, a);
@@ -332,9 +332,10 @@ __global__ void arm_kernel(CavityRun* runs, const int* __restrict__ slot_list, i
 // ---------------------------------------------------------------------------
 template <class P, int TY, int SCHEME = 0>
 struct TileKernel {
-    static constexpr int NT = TileThreads<P, TY>::value;
-    static constexpr size_t smem = sizeof(TileSmem<P, kTileX, TY, NT>);
-    static constexpr auto fn = step_kernel<P, kTileX, TY, NT, SCHEME>;
+    static constexpr int TX = tile_width(sizeof(typename P::R) == 8 ? 0 : 1, TY);
+    static constexpr int NT = TileThreads<P, TX, TY>::value;
+    static constexpr size_t smem = sizeof(TileSmem<P, TX, TY, NT>);
+    static constexpr auto fn = step_kernel<P, TX, TY, NT, SCHEME>;
     static cudaError_t prepare()
     {
         cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
