@@ -171,7 +171,7 @@ struct Smem3 {
     R yl[7][TY + 1];
     R xisn[BX], xdtw[BX];   // CellLine is_next, dt_w of the ringed tile
     R yisn[BY], ydtw[BY];
-    double red[NT / 32][4];
+    double red[NT / 32][4];  // per-warp residual partials
     int plan[3];  // after the stop test: done, cur, sum slot
 };
 
@@ -593,27 +593,10 @@ __global__ void __launch_bounds__(TX* TY) step3_kernel(const Desc3* __restrict__
     }
     if (bad) s0 = R(NAN);
     // residual sums: warp sums in the working precision, warps and units in FP64
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        s0 += __shfl_xor_sync(0xffffffffu, s0, o);
-        s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-        s2 += __shfl_xor_sync(0xffffffffu, s2, o);
-        s3 += __shfl_xor_sync(0xffffffffu, s3, o);
-    }
-    if ((tid & 31) == 0) {
-        sm.red[tid >> 5][0] = (double)s0;
-        sm.red[tid >> 5][1] = (double)s1;
-        sm.red[tid >> 5][2] = (double)s2;
-        sm.red[tid >> 5][3] = (double)s3;
-    }
+    const R sum = rtlbfs::warp_sum4(s0, s1, s2, s3);
+    if ((tid & 7) == 0) sm.red[tid >> 5][(tid & 31) >> 3] = (double)sum;
     __syncthreads();
-    if (tid == 0) {
-        double a[4] = {0.0, 0.0, 0.0, 0.0};
-        for (int w = 0; w < NT / 32; ++w)
-            for (int q = 0; q < 4; ++q) a[q] += sm.red[w][q];
-        // the step's residual sums; the next launch tests them
-        for (int q = 0; q < 4; ++q) atomicAdd(&run->acc[slot3][q], a[q]);
-    }
+    rtlbfs::add_sums(sm.red, NT / 32, run->acc[slot3]);  // the next launch tests them
 }
 
 // ---------------------------------------------------------------------------

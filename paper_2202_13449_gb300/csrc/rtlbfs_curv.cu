@@ -587,36 +587,10 @@ __global__ void __launch_bounds__(TX* TY) curv_step_kernel(const DescC* __restri
         s3 = T1 * T1;
     }
     if (bad) s0 = R(NAN);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        s0 += __shfl_xor_sync(0xffffffffu, s0, o);
-        s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-        s2 += __shfl_xor_sync(0xffffffffu, s2, o);
-        s3 += __shfl_xor_sync(0xffffffffu, s3, o);
-    }
-    if ((tid & 31) == 0) {
-        sm.red[tid >> 5][0] = s0;
-        sm.red[tid >> 5][1] = s1;
-        sm.red[tid >> 5][2] = s2;
-        sm.red[tid >> 5][3] = s3;
-    }
+    const R sum = rtlbfs::warp_sum4(s0, s1, s2, s3);
+    if ((tid & 7) == 0) sm.red[tid >> 5][(tid & 31) >> 3] = sum;
     __syncthreads();
-    // warp 0 adds the warp partials in the arithmetic type (a serial FP64
-    // loop would hold GB300's narrow FP64 pipe at the tail of every block);
-    // the tile sums go to the FP64 sums across tiles
-    double acc4[4];
-    if (tid < 32) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            R v = tid < NT / 32 ? sm.red[tid][q] : R(0);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            acc4[q] = (double)v;
-        }
-    }
-    // the step's residual sums; the next launch tests them
-    if (tid == 0)
-        for (int q = 0; q < 4; ++q) atomicAdd(&run->acc[slot3][q], acc4[q]);
+    rtlbfs::add_sums(sm.red, NT / 32, run->acc[slot3]);  // the next launch tests them
 }
 
 // ---------------------------------------------------------------------------

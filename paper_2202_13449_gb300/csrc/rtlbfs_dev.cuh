@@ -13,6 +13,7 @@
 
 #include <cmath>
 #include <cstdint>
+#include <cstring>
 
 namespace rtlbfs {
 
@@ -147,17 +148,59 @@ __host__ __device__ inline double r12(double num, double den)
     return den > 0.0 ? sqrt(num) / sqrt(den) : INFINITY;
 }
 
-// r12(num, den) < tol, decided without the FP64 square roots and division
-// unless the ratio lies within 2 % of tol^2: the same outcome as the
-// formula (its rounding error is ~1e-16 relative), a fraction of its
-// latency on the narrow FP64 units of this GPU.
+// The two words of a double, and tests on them.  The stop test stands at the
+// head of every step kernel's chain, and an FP64 operation there takes about
+// as long as twenty integer ones (an FP64 comparison too).  With the sums of
+// warp_sum4 and add_sums below: 512^2 10.95 -> 10.40 us per step, 1024x512
+// 21.6 -> 19.2, 301x203 6.75 -> 6.30, 64^2 6.5 -> 5.95.
+__host__ __device__ inline unsigned hi_word(double x)
+{
+#ifdef __CUDA_ARCH__
+    return (unsigned)__double2hiint(x);
+#else
+    unsigned long long u;
+    std::memcpy(&u, &x, sizeof(u));
+    return (unsigned)(u >> 32);
+#endif
+}
+__host__ __device__ inline unsigned lo_word(double x)
+{
+#ifdef __CUDA_ARCH__
+    return (unsigned)__double2loint(x);
+#else
+    unsigned long long u;
+    std::memcpy(&u, &x, sizeof(u));
+    return (unsigned)u;
+#endif
+}
+__host__ __device__ inline bool nan_bits(double x)
+{
+    const unsigned h = hi_word(x) & 0x7fffffffu;
+    return h > 0x7ff00000u || (h == 0x7ff00000u && lo_word(x) != 0);
+}
+__host__ __device__ inline bool pos_inf_bits(double x)
+{
+    return hi_word(x) == 0x7ff00000u && lo_word(x) == 0;
+}
+
+// r12(num, den) < tol, decided without FP64 arithmetic unless the ratio lies
+// near tol^2: the same outcome as the formula.  The high word of a positive
+// normal double is a fixed-point logarithm, log2 x = 1023 less than hi / 2^20
+// and up to 0.0861 more (the mantissa's chord), so num and tol^2 den compare
+// by their words outside a band of 0.27 in log2.
 __host__ __device__ inline bool r12_below(double num, double den, double tol)
 {
-    if (!(den > 0.0) || !(tol > 0.0)) return false;
-    const double q = tol * tol * den;
-    if (q >= 2.2250738585072014e-308 && q < 1e300) {
-        if (num < 0.98 * q) return true;
-        if (num > 1.02 * q) return false;
+    const unsigned ht = hi_word(tol), hd = hi_word(den), hn = hi_word(num);
+    // tol <= 0 (a set sign, or zero), or den <= 0
+    if ((ht >> 31) || (ht | lo_word(tol)) == 0) return false;
+    if ((hd >> 31) || (hd | lo_word(den)) == 0) return false;
+    auto normal = [](unsigned h) { return h >= 0x00100000u && h < 0x7ff00000u; };
+    if (normal(ht) && normal(hd) && normal(hn)) {
+        constexpr int bias = 1023 << 20, chord = 90400;  // 0.0861 in 2^-20, rounded up
+        // half units: the sum of three words leaves 32 bits
+        const int n = ((int)hn - bias) / 2, q = ((int)ht - bias) + ((int)hd - bias) / 2;
+        if (n + chord / 2 + 2 < q) return true;
+        if (n > q + 3 * chord / 2 + 2) return false;
     }
     return r12(num, den) < tol;
 }
@@ -176,9 +219,9 @@ __host__ __device__ inline CavityCtl stop_test(CavityCtl c, const double s[4])
     c.steps += 1;
     c.cur ^= 1;
     c.pend = 0;
-    // r12 is NaN exactly when num is NaN or both are infinite (den > 0)
-    const bool nan_u = isnan(su) || (du > 0.0 && isinf(su) && isinf(du));
-    const bool nan_T = isnan(sT) || (dT > 0.0 && isinf(sT) && isinf(dT));
+    // r12 is NaN exactly when num is NaN or both are infinite (sums of squares)
+    const bool nan_u = nan_bits(su) || (pos_inf_bits(su) && pos_inf_bits(du));
+    const bool nan_T = nan_bits(sT) || (pos_inf_bits(sT) && pos_inf_bits(dT));
     int status = kRunning;
     if (nan_u || nan_T) status = kDiverged;
     else if (r12_below(su, du, c.tol) && r12_below(sT, dT, c.tol)) status = kConverged;
@@ -204,6 +247,35 @@ __device__ inline CavityCtl run_head(const CavityRun* r, int par)
 #pragma unroll
     for (int q = 0; q < 4; ++q) s[q] = slot == 0 ? a[0][q] : (slot == 1 ? a[1][q] : a[2][q]);
     return stop_test(c, s);
+}
+
+// Sums of four values over a warp: lane l gets the sum of value l / 8.  Half
+// the values change lanes in each of the first two steps, so six shuffles do
+// what twenty would.
+template <typename R>
+__device__ __forceinline__ R warp_sum4(R a0, R a1, R a2, R a3)
+{
+    const unsigned all = 0xffffffffu;
+    const bool h16 = (threadIdx.x & 16) != 0, h8 = (threadIdx.x & 8) != 0;
+    const R b0 = (h16 ? a2 : a0) + __shfl_xor_sync(all, h16 ? a0 : a2, 16);
+    const R b1 = (h16 ? a3 : a1) + __shfl_xor_sync(all, h16 ? a1 : a3, 16);
+    R c = (h8 ? b1 : b0) + __shfl_xor_sync(all, h8 ? b0 : b1, 8);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) c += __shfl_xor_sync(all, c, o);
+    return c;
+}
+
+// A block's residual sums from its warps' partials red[warp][q], in the
+// order of the warps: thread q < 4 adds sum q to the step's in FP64 (four
+// conversions and atomics at once, not one after the other).
+template <typename R>
+__device__ __forceinline__ void add_sums(const R (*red)[4], int warps, double* acc)
+{
+    if (threadIdx.x < 4) {
+        R v = R(0);
+        for (int w = 0; w < warps; ++w) v += red[w][threadIdx.x];
+        atomicAdd(&acc[threadIdx.x], (double)v);
+    }
 }
 
 // What the cavity's first unit of a launch of parity par writes: the

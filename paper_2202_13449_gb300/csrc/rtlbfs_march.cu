@@ -122,14 +122,6 @@ __device__ __forceinline__ Vec4<R> shfl_dn1(const Vec4<R>& v)
     return {shfl_dn1(v.x), shfl_dn1(v.y), shfl_dn1(v.z), shfl_dn1(v.w)};
 }
 
-template <typename R>
-__device__ __forceinline__ R wsum(R v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
 }  // namespace
 
 template <class P>
@@ -344,18 +336,9 @@ march_kernel(const CavityDesc* __restrict__ descs, CavityRun* __restrict__ runs,
             gy0 = gy1;
         }
         if (bad) s0 = R(NAN);
-        s0 = wsum(s0);
-        s1 = wsum(s1);
-        s2 = wsum(s2);
-        s3 = wsum(s3);
+        const R sum = warp_sum4(s0, s1, s2, s3);
         // the step's residual sums; the next launch tests them
-        if (lane == 0) {
-            double* acc = run->acc[slot3];
-            atomicAdd(&acc[0], (double)s0);
-            atomicAdd(&acc[1], (double)s1);
-            atomicAdd(&acc[2], (double)s2);
-            atomicAdd(&acc[3], (double)s3);
-        }
+        if ((lane & 7) == 0) atomicAdd(&run->acc[slot3][lane >> 3], (double)sum);
         __syncwarp();
     }
 }

@@ -517,21 +517,9 @@ march2_kernel(const CavityDesc* __restrict__ descs, CavityRun* __restrict__ runs
             }
         }
         float a0 = bad ? NAN : s0.x + s0.y, a1 = s1.x + s1.y, a2 = s2.x + s2.y, a3 = s3.x + s3.y;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            a0 += __shfl_xor_sync(0xffffffffu, a0, o);
-            a1 += __shfl_xor_sync(0xffffffffu, a1, o);
-            a2 += __shfl_xor_sync(0xffffffffu, a2, o);
-            a3 += __shfl_xor_sync(0xffffffffu, a3, o);
-        }
+        const float sum = warp_sum4(a0, a1, a2, a3);
         // the step's residual sums; the next launch tests them
-        if (lane == 0) {
-            double* acc = run->acc[slot3];
-            atomicAdd(&acc[0], (double)a0);
-            atomicAdd(&acc[1], (double)a1);
-            atomicAdd(&acc[2], (double)a2);
-            atomicAdd(&acc[3], (double)a3);
-        }
+        if ((lane & 7) == 0) atomicAdd(&run->acc[slot3][lane >> 3], (double)sum);
         __syncwarp();
     }
 }

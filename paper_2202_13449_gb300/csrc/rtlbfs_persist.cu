@@ -153,11 +153,10 @@ persist_kernel(const CavityDesc* __restrict__ dp, CavityCtl* __restrict__ ctl,
                                          static_cast<const Vec4<S>*>(dp->f[rb][0]),
                                          static_cast<Vec4<S>*>(dp->f[rb ^ 1][0]), true);
         __syncthreads();
-        double a[4];
-        if (tid < 32) tile_sums(sm, a);
+        double* acc = pc->acc[k % 3];
+        tile_sums(sm, acc);  // threads 0-3
+        if (tid < 32) __syncwarp();
         if (tid == 0) {
-            double* acc = pc->acc[k % 3];
-            for (int q = 0; q < 4; ++q) atomicAdd(&acc[q], a[q]);
             __threadfence();  // the tile's new state (all threads, before the barrier) and sums
             if (t != withhold) st_release(&tstep[t], k);
             const unsigned prev = atomicAdd(&pc->arrive[k % 3], 1u);

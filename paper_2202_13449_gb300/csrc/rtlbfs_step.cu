@@ -78,11 +78,7 @@ step_kernel(const CavityDesc* __restrict__ descs, CavityRun* __restrict__ runs,
                                                static_cast<const Vec4<S>*>(dp->f[cur][0]),
                                                static_cast<Vec4<S>*>(dp->f[cur ^ 1][0]), first);
         __syncthreads();
-        double a[4];
-        if (tid < 32) tile_sums(sm, a);
-        // the step's residual sums; the next launch tests them
-        if (tid == 0)
-            for (int q = 0; q < 4; ++q) atomicAdd(&run->acc[slot3][q], a[q]);
+        tile_sums(sm, run->acc[slot3]);  // the next launch tests them
         __syncthreads();
     }
 }

@@ -38,7 +38,7 @@ struct TileSmem {
     FaceLine<R> yl[TY + 1];
     CellLine<R> xc[BX];
     CellLine<R> yc[BY];
-    R red[NT / 32][4];  // per-warp residual partials (tile_sums adds them)
+    R red[NT < 32 ? 1 : NT / 32][4];  // per-warp residual partials (tile_sums adds them)
     CavityDesc desc;  // the tile's cavity, staged by stage_tile
     int plan[3];      // the tile's step after its cavity's stop test: done, cur, sum slot
     int last;         // persistent kernel: this block finalises the step
@@ -296,28 +296,13 @@ struct FlatTile {
     static constexpr bool value = sizeof(typename P::R) == 8 && TX == 16 && TY == 2;
 };
 
-// The tile's four residual sums from the per-warp partials in sm.red:
-// warp 0 adds them in the arithmetic type (shuffles; on GB300 an FP64
-// instruction occupies the narrow FP64 pipe for 16 cycles, so a serial FP64
-// loop here lengthened every block's tail) and returns them in FP64, the
-// precision of the sums across tiles.  Call from all of warp 0, after the
-// barrier that follows tile_step.
+// The tile's residual sums added to the step's, from the per-warp partials
+// in sm.red (one row for the flat tile).  Call after the barrier that
+// follows the tile's step.
 template <class P, int TX, int TY, int NT>
-__device__ __forceinline__ void tile_sums(const TileSmem<P, TX, TY, NT>& sm, double a[4])
+__device__ __forceinline__ void tile_sums(const TileSmem<P, TX, TY, NT>& sm, double* acc)
 {
-    using R = typename P::R;
-    if constexpr (FlatTile<P, TX, TY>::value) {  // already the tile's sums
-#pragma unroll
-        for (int q = 0; q < 4; ++q) a[q] = sm.red[0][q];
-        return;
-    }
-    const int lane = threadIdx.x & 31;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        R v = lane < NT / 32 ? sm.red[lane][q] : R(0);
-        v = warp_sum(v);
-        a[q] = (double)v;
-    }
+    add_sums(sm.red, FlatTile<P, TX, TY>::value ? 1 : NT / 32, acc);
 }
 
 // One tile of one time step on cavity *dp, tile origin (i0, j0): phases 1-4
@@ -619,16 +604,8 @@ __device__ __forceinline__ void tile_step(TileSmem<P, TX, TY, NT>& sm, const Cav
         if (bad) s0 = R(NAN);
     }
     // warp sums in R, then FP64 across warps and tiles
-    s0 = warp_sum(s0);
-    s1 = warp_sum(s1);
-    s2 = warp_sum(s2);
-    s3 = warp_sum(s3);
-    if ((tid & 31) == 0) {
-        sm.red[tid >> 5][0] = s0;
-        sm.red[tid >> 5][1] = s1;
-        sm.red[tid >> 5][2] = s2;
-        sm.red[tid >> 5][3] = s3;
-    }
+    const R sum = warp_sum4(s0, s1, s2, s3);
+    if ((tid & 7) == 0) sm.red[tid >> 5][(tid & 31) >> 3] = sum;
 }
 
 // tile_step for the 16 x 2 FP64 tile (RTLBFS), one phase item per thread.
