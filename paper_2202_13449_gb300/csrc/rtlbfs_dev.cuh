@@ -422,7 +422,7 @@ struct CellNT {
 // Only differences of some of these enter; they are formed as such (one FMA
 // chain from the negated left column), and the middle column's slopes enter
 // doubled (D = 2 s_0 = s_-1 + s_+1), the powers of two going into constants:
-// 156 operations a face where forming each term by itself takes 172.  (In
+// 153 operations a face where forming each term by itself takes 172.  (In
 // FP64 the step runs at the FMA rate: 40 steps of a 400^2 mesh 8.44 -> 8.15 ms;
 // FP32 512^2 11.46 -> 11.26 ms for 1000 steps.)
 //
@@ -471,8 +471,7 @@ __host__ __device__ __forceinline__ void face_flux_wall(const V A[4], const V Na
     const V TA = Tbar + A[3], TM = Tbar + M[3], TB = Tbar + B[3];
     const V mnA = vfma(A[0], A[1], A[1]), mnM = vfma(M[0], M[1], M[1]), mnB = vfma(B[0], B[1], B[1]);
     const V mtA = vfma(A[0], A[2], A[2]), mtM = vfma(M[0], M[2], M[2]), mtB = vfma(B[0], B[2], B[2]);
-    const V PnnA = mnA * A[1], PnnM = mnM * M[1], PnnB = mnB * B[1];
-    const V PntM = mnM * M[2], QnM = mnM * TM;
+    const V PnnM = mnM * M[1], PntM = mnM * M[2], QnM = mnM * TM;
     const V eA = vfma(A[0], TA, A[3]), eM = vfma(M[0], TM, M[3]), eB = vfma(B[0], TB, B[3]);
     // column a = 0 in b: rho = rM + b sd, u_n = M1 + b sn, u_t = M2 + b st,
     // T = TM + b sT with (sd, sn, st, sT) = D / 2.  The names' last digit is
@@ -499,14 +498,14 @@ __host__ __device__ __forceinline__ void face_flux_wall(const V A[4], const V Na
     const V dx_Pnt = vfma(mnB, B[2], nmnA * A[2]), dx_Q = vfma(mnB, TB, nmnA * TA);
     const V dxx_mn = vfma(m2, mnM, mnB + mnA), dxx_mt = vfma(m2, mtM, mtB + mtA);
     const V dxx_e = vfma(m2, eM, eB + eA), dxx_dr = vfma(m2, M[0], B[0] + A[0]);
-    const V dxx_Pnn = vfma(m2, PnnM, PnnB + PnnA);
 
     // Eq. 46: drho* = rho* - 1
-    const V drs = vfma(half, (dxx_Pnn - dx_mn) + dPnt_o,
+    const V dxx_Pnn = vfma(mnB, B[1], vfma(mnA, A[1], vfma(m2, PnnM, dPnt_o - dx_mn)));  // and those
+    const V drs = vfma(half, dxx_Pnn,
                        vfma(hcs2, dxx_dr, vfma(quarter, Ptt_q4, vfma(mhalf, mt_l2, M[0]))));
     // Eq. 47: (rho u_n)*, (rho u_t)*
     V mns_ = vfma(hcs2, vfma(three, dxx_mn, vfma(half, mn_q4, dmt_o)),
-                  vfma(mhalf, vfma(cs2, dx_dr, PnnB - PnnA) + Pnt_o2, mnM));
+                  vfma(mhalf, vfma(cs2, dx_dr, vfma(mnB, B[1], vfma(nmnA, A[1], Pnt_o2))), mnM));
     V mts_ = vfma(hcs2, vfma(T::bc(1.5), mt_q4, dxx_mt + (mnB_o + nmnA_o)),
                   vfma(mhalf, dx_Pnt + Ptt_o2, vfma(mhcs2, D[0], mtM)));
     // Eq. 48: (rho T)* - Tbar
@@ -554,108 +553,6 @@ __host__ __device__ __forceinline__ void face_flux(const CellNT<V>& L, const Cel
     face_flux_columns<V>(A, Na, M, D, B, Sb, Tbar, fl, keep, u_wall, F);
 }
 
-// Green-Gauss gradients of a cell p from its four neighbours in the
-// CellLine form of Eqs. 55-56 (ixe = is_next of the cell, ixw that of its
-// west neighbour; iyn, iys along y), FP32, two components per packed
-// FP32x2 instruction:
-//   g_x = (e - p) ixe + (p - w) ixw,  g_y = (n - p) iyn + (p - s) iys.
-__device__ __forceinline__ void gg_gradient_f32(const Vec4<float>& p, const Vec4<float>& e,
-                                                const Vec4<float>& w, const Vec4<float>& n,
-                                                const Vec4<float>& s, float ixe, float ixw,
-                                                float iyn, float iys, Vec4<float>& gx,
-                                                Vec4<float>& gy)
-{
-    const float2 m1 = make_float2(-1.0f, -1.0f);
-    const float2 xe = make_float2(ixe, ixe), xw = make_float2(ixw, ixw);
-    const float2 yn = make_float2(iyn, iyn), ys = make_float2(iys, iys);
-    const float2 P[2] = {make_float2(p.x, p.y), make_float2(p.z, p.w)};
-    const float2 E[2] = {make_float2(e.x, e.y), make_float2(e.z, e.w)};
-    const float2 W[2] = {make_float2(w.x, w.y), make_float2(w.z, w.w)};
-    const float2 N[2] = {make_float2(n.x, n.y), make_float2(n.z, n.w)};
-    const float2 S[2] = {make_float2(s.x, s.y), make_float2(s.z, s.w)};
-    float2 gxp[2], gyp[2];
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        // a - b as fma(b, -1, a): exact, one rounding like the subtraction
-        gxp[i] = __ffma2_rn(__ffma2_rn(P[i], m1, E[i]), xe, __fmul2_rn(__ffma2_rn(W[i], m1, P[i]), xw));
-        gyp[i] = __ffma2_rn(__ffma2_rn(P[i], m1, N[i]), yn, __fmul2_rn(__ffma2_rn(S[i], m1, P[i]), ys));
-    }
-    gx = {gxp[0].x, gxp[0].y, gxp[1].x, gxp[1].y};
-    gy = {gyp[0].x, gyp[0].y, gyp[1].x, gyp[1].y};
-}
-
-// Flux balance of a cell, FP32, in packed pairs (mass, x-momentum) and
-// (y-momentum, energy): div = ax (F_e - F_w) + ay (F_n - F_s), ax and ay the
-// time step over the cell's widths.
-__device__ __forceinline__ void flux_div_f32(const Vec4<float>& Fw, const Vec4<float>& Fe,
-                                             const Vec4<float>& Fs, const Vec4<float>& Fn, float ax,
-                                             float ay, float& d0, float& d1, float& d2, float& d3)
-{
-    const float2 m1 = make_float2(-1.0f, -1.0f);
-    const float2 ax2 = make_float2(ax, ax), ay2 = make_float2(ay, ay);
-    const float2 d01 = __ffma2_rn(
-        __ffma2_rn(make_float2(Fw.x, Fw.y), m1, make_float2(Fe.x, Fe.y)), ax2,
-        __fmul2_rn(__ffma2_rn(make_float2(Fs.x, Fs.y), m1, make_float2(Fn.x, Fn.y)), ay2));
-    const float2 d23 = __ffma2_rn(
-        __ffma2_rn(make_float2(Fw.z, Fw.w), m1, make_float2(Fe.z, Fe.w)), ax2,
-        __fmul2_rn(__ffma2_rn(make_float2(Fs.z, Fs.w), m1, make_float2(Fn.z, Fn.w)), ay2));
-    d0 = d01.x;
-    d1 = d01.y;
-    d2 = d23.x;
-    d3 = d23.y;
-}
-
-// face_columns in FP32 from the two cells' working values (rho - 1, u, v,
-// T - Tz) and their gradients along the face normal (gn) and tangent (gt),
-// all in storage order, two components per packed FP32x2 instruction: the
-// pairs (rho, u) and (v, T) of a record sit in adjacent registers.  The
-// operations of face_columns on the face-frame cells of face_cells; ISX: x-face (n = x), else y-face (n = y: u_n = v, u_t = u).
-template <bool ISX>
-__device__ __forceinline__ void face_columns_f32(const Vec4<float>& vl, const Vec4<float>& vr,
-                                                 const Vec4<float>& gnl, const Vec4<float>& gtl,
-                                                 const Vec4<float>& gnr, const Vec4<float>& gtr,
-                                                 const FaceLine<float>& fl, float A[4],
-                                                 float Na[4], float M[4], float D[4], float B[4],
-                                                 float Sb[4])
-{
-    const float h = fl.h;
-    const float wL = fl.cL + h, mwR = fl.cR - h;
-    const float2 cL2 = make_float2(fl.cL, fl.cL), cR2 = make_float2(fl.cR, fl.cR);
-    const float2 wL2 = make_float2(wL, wL), mwR2 = make_float2(mwR, mwR);
-    const float2 h2 = make_float2(h, h), mh2 = make_float2(-h, -h), half2 = make_float2(0.5f, 0.5f);
-    const float2 m1 = make_float2(-1.0f, -1.0f);
-    // the left cell's temperature is carried by Tbar = Tz + T_L
-    const float2 ql[2] = {make_float2(vl.x, vl.y), make_float2(vl.z, 0.0f)};
-    const float2 qr[2] = {make_float2(vr.x, vr.y), make_float2(vr.z, vr.w - vl.w)};
-    const float2 nl[2] = {make_float2(gnl.x, gnl.y), make_float2(gnl.z, gnl.w)};
-    const float2 tl[2] = {make_float2(gtl.x, gtl.y), make_float2(gtl.z, gtl.w)};
-    const float2 nr[2] = {make_float2(gnr.x, gnr.y), make_float2(gnr.z, gnr.w)};
-    const float2 tr[2] = {make_float2(gtr.x, gtr.y), make_float2(gtr.z, gtr.w)};
-    float2 a[2], na[2], m[2], d2[2], b[2], sb[2];
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        a[i] = __ffma2_rn(nl[i], cL2, ql[i]);
-        na[i] = __fmul2_rn(tl[i], mh2);
-        b[i] = __ffma2_rn(nr[i], cR2, qr[i]);
-        sb[i] = __fmul2_rn(tr[i], h2);
-        m[i] = __fmul2_rn(half2, __fadd2_rn(__ffma2_rn(nl[i], wL2, ql[i]), __ffma2_rn(nr[i], mwR2, qr[i])));
-        d2[i] = __ffma2_rn(na[i], m1, sb[i]);
-    }
-    // face-frame order: (rho, u_n, u_t, T)
-    auto put = [](const float2* v, float* d) {
-        d[0] = v[0].x;
-        d[1] = ISX ? v[0].y : v[1].x;
-        d[2] = ISX ? v[1].x : v[0].y;
-        d[3] = v[1].y;
-    };
-    put(a, A);
-    put(na, Na);
-    put(m, M);
-    put(d2, D);
-    put(b, B);
-    put(sb, Sb);
-}
-
 // The original TLBFS face stage (Section 2.2), from the same inputs as
 // face_flux and in the same frame: (a) D2Q9 equilibria (Eqs. 3-4, c_p = 1)
 // at the nodes x_S - e_i h, i.e. node (a, b) = -e_i of the column form
@@ -666,21 +563,24 @@ __device__ __forceinline__ void face_columns_f32(const Vec4<float>& vl, const Ve
 // constants cancel in every moment used except the pressure c_s^2, which is
 // dropped from the normal momentum flux as in face_flux.  The Dirichlet
 // override of (rho T)* is omitted: it enters no flux (u*_n = 0 there).
-template <typename V>
-__host__ __device__ __forceinline__ void face_flux_tlbfs(const CellNT<V>& L, const CellNT<V>& Rc,
-                                                        V Tbar, const FaceLine<V>& fl, V keep,
-                                                        V u_wall, V F[4])
+//
+// A flux is sum_i e_in e_ia [f*_i + (1/2 - tau) (f*_i - f_i)]: the moments
+// of the predicted state's equilibria are c_s^2 rho + rho u_n u_n, rho u_n
+// u_t and rho u_n T exactly, so only the nodes' equilibria are formed one by
+// one, without their weights, and summed by weight and sign: 230 operations
+// a face where the equilibria of both states take 330 (512^2 FP32 14.7 -> 12.7 us
+// per step, FP64 492 -> 368).
+template <typename V, class W>
+__host__ __device__ __forceinline__ void face_flux_tlbfs_wall(const CellNT<V>& L, const CellNT<V>& Rc,
+                                                             V Tbar, const FaceLine<V>& fl, W wall,
+                                                             V F[4])
 {
     using T = vtraits<V>;
-    const V half = T::bc(0.5), one = T::bc(1.0), three = T::bc(3.0);
-    const V c45 = T::bc(4.5), c15 = T::bc(1.5);
-    // D2Q9 in the face frame (n, t); weights of Eq. 6
-    constexpr int en[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1};
-    constexpr int et[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
+    const V half = T::bc(0.5), one = T::bc(1.0), c45 = T::bc(4.5), mc15 = T::bc(-1.5);
+    const V cs2 = T::bc(1.0 / 3.0);
     const V w0 = T::bc(4.0 / 9.0), w1 = T::bc(1.0 / 9.0), w2 = T::bc(1.0 / 36.0);
     const V h = fl.h;
     const V wL = fl.cL + h, mwR = fl.cR - h;
-    const V hh = h * half;
     // columns a = -1 (left plane), 0 (mean), +1 (right plane): value + b slope
     V C[3][4], Sl[3][4];
 #pragma unroll
@@ -690,68 +590,79 @@ __host__ __device__ __forceinline__ void face_flux_tlbfs(const CellNT<V>& L, con
         C[2][k] = vfma(Rc.gn[k], fl.cR, Rc.q[k]);
         Sl[2][k] = Rc.gt[k] * h;
         C[1][k] = half * (vfma(L.gn[k], wL, L.q[k]) + vfma(Rc.gn[k], mwR, Rc.q[k]));
-        Sl[1][k] = hh * (L.gt[k] + Rc.gt[k]);
+        Sl[1][k] = half * (Sl[0][k] + Sl[2][k]);
     }
-    // (a), (b): equilibria at the nodes and their moments
-    V df[9], dg[9];
-    V drs = T::bc(0.0), mn = T::bc(0.0), mt = T::bc(0.0), es = T::bc(0.0);
-#pragma unroll
-    for (int i = 0; i < 9; ++i) {
-        const int a = 1 - en[i], b = -et[i];  // column index, offset along t
+    // (a) equilibria of direction (en, et) at the node (-en, -et), over their
+    // weights: f_i / w_i - 1 = drho + rho (3 eu + 4.5 eu^2 - 1.5 u^2), and
+    // g_i / w_i - Tbar from rho T - Tbar = tau + drho T
+    auto equil = [&](int en, int et, V& f, V& g) {
+        const int a = 1 - en;
         V q[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k)
-            q[k] = b == 0 ? C[a][k] : (b > 0 ? C[a][k] + Sl[a][k] : C[a][k] - Sl[a][k]);
-        const V w = i == 0 ? w0 : (i < 5 ? w1 : w2);
-        V eu = T::bc(0.0);
-        if (en[i] > 0) eu = eu + q[1];
-        if (en[i] < 0) eu = eu - q[1];
-        if (et[i] > 0) eu = eu + q[2];
-        if (et[i] < 0) eu = eu - q[2];
-        const V usq = vfma(q[1], q[1], q[2] * q[2]);
-        const V rho = one + q[0];
-        // f_i - w_i = w_i (drho + rho (3 eu + 4.5 eu^2 - 1.5 u^2))
-        df[i] = w * vfma(rho, vfma(eu, vfma(c45, eu, three), T::bc(0.0) - c15 * usq), q[0]);
-        // rho T - Tbar = tau + drho T at the node; g_i - w_i Tbar
-        const V e_node = vfma(q[0], Tbar + q[3], q[3]);
-        dg[i] = w * vfma(three * eu, Tbar + e_node, e_node);
-        drs = drs + df[i];
-        if (en[i] > 0) mn = mn + df[i];
-        if (en[i] < 0) mn = mn - df[i];
-        if (et[i] > 0) mt = mt + df[i];
-        if (et[i] < 0) mt = mt - df[i];
-        es = es + dg[i];
-    }
+            q[k] = et == 0 ? C[a][k] : (et < 0 ? C[a][k] + Sl[a][k] : C[a][k] - Sl[a][k]);
+        const V e = vfma(q[0], Tbar + q[3], q[3]);
+        const V u2 = mc15 * vfma(q[1], q[1], q[2] * q[2]);
+        if (en == 0 && et == 0) {
+            f = vfma(one + q[0], u2, q[0]);
+            g = e;
+            return;
+        }
+        // eu = sign * s with s one velocity, or the sum or difference of both
+        const V s = et == 0 ? q[1] : (en == 0 ? q[2] : (en == et ? q[1] + q[2] : q[1] - q[2]));
+        const V three = T::bc((en != 0 ? en : et) > 0 ? 3.0 : -3.0);
+        f = vfma(one + q[0], vfma(s, vfma(c45, s, three), u2), q[0]);
+        g = vfma(three * s, Tbar + e, e);
+    };
+    // (b) the predicted variables as moments, with those of the fluxes:
+    // sums over the directions of one weight, by sign
+    V f0, g0, fp, gp, fm, gm;
+    equil(0, 0, f0, g0);
+    equil(1, 0, fp, gp);
+    equil(-1, 0, fm, gm);
+    const V Sn = fp + fm, Dn = fp - fm, Gn = gp + gm, En = gp - gm;
+    equil(0, 1, fp, gp);
+    equil(0, -1, fm, gm);
+    const V S1 = Sn + (fp + fm), Dt = fp - fm, G1 = Gn + (gp + gm);
+    V fpp, gpp, fmm, gmm;
+    equil(1, 1, fpp, gpp);
+    equil(-1, -1, fmm, gmm);
+    const V Sa = fpp + fmm, Da = fpp - fmm, Ga = gpp + gmm, Ea = gpp - gmm;
+    equil(1, -1, fp, gp);
+    equil(-1, 1, fm, gm);
+    const V Sb = fp + fm, Db = fp - fm, Gb = gp + gm, Eb = gp - gm;
+    const V S2 = Sa + Sb;
+    const V drs = vfma(w0, f0, vfma(w1, S1, w2 * S2));
+    V mn = vfma(w1, Dn, w2 * (Da + Db));
+    V mt = vfma(w1, Dt, w2 * (Da - Db));
+    const V es = vfma(w0, g0, vfma(w1, G1, w2 * (Ga + Gb)));
+    const V Xnn = vfma(w1, Sn, w2 * S2), Xnt = w2 * (Sa - Sb), Qn = vfma(w1, En, w2 * (Ea + Eb));
     const V rho_s = one + drs;
-    mn = mn * keep;
-    mt = vfma(keep, mt, (one - keep) * (rho_s * u_wall));
+    wall(mn, mt, rho_s);
     const V inv = T::rcp(rho_s);
     const V uns = mn * inv, uts = mt * inv;
-    const V usq_s = vfma(uns, uns, uts * uts);
-    // (c) fluxes along +n with the non-equilibrium parts; 1/2 - tau_f =
-    // -3 nu / h = 6 (-nu / 2h), likewise for tau_g (Eqs. 9-10)
-    const V six = T::bc(6.0);
-    const V cf = six * fl.m_nu_2h, cg = six * fl.m_chi_2h;
-    V Fnn = T::bc(0.0), Fnt = T::bc(0.0), Q = T::bc(0.0);
-#pragma unroll
-    for (int i = 0; i < 9; ++i) {
-        if (en[i] == 0) continue;  // no flux along n
-        const V w = i < 5 ? w1 : w2;
-        V eu = en[i] > 0 ? uns : T::bc(0.0) - uns;
-        if (et[i] > 0) eu = eu + uts;
-        if (et[i] < 0) eu = eu - uts;
-        const V dfs = w * vfma(rho_s, vfma(eu, vfma(c45, eu, three), T::bc(0.0) - c15 * usq_s), drs);
-        const V dgs = w * vfma(three * eu, Tbar + es, es);
-        const V pf = vfma(cf, dfs - df[i], dfs);  // f* + (1/2 - tau_f)(f* - f_node)
-        const V pg = vfma(cg, dgs - dg[i], dgs);
-        Fnn = Fnn + pf;  // e_n^2 = 1
-        if (et[i] != 0) Fnt = (en[i] * et[i] > 0) ? Fnt + pf : Fnt - pf;
-        Q = en[i] > 0 ? Q + pg : Q - pg;
-    }
+    // (c) fluxes along +n: the moments of the predicted equilibria plus the
+    // non-equilibrium parts; 1/2 - tau_f = -3 nu / h = 6 (-nu / 2h), likewise
+    // for tau_g (Eqs. 9-10)
+    const V cf = T::bc(6.0) * fl.m_nu_2h, cg = T::bc(6.0) * fl.m_chi_2h;
+    const V Fnn = vfma(mn, uns, cs2 * drs), Fnt = mn * uts, Q = uns * (Tbar + es);
     F[0] = mn;
-    F[1] = Fnn;
-    F[2] = Fnt;
-    F[3] = Q;
+    F[1] = vfma(cf, Fnn - Xnn, Fnn);
+    F[2] = vfma(cf, Fnt - Xnt, Fnt);
+    F[3] = vfma(cg, Q - Qn, Q);
+}
+
+template <typename V>
+__host__ __device__ __forceinline__ void face_flux_tlbfs(const CellNT<V>& L, const CellNT<V>& Rc,
+                                                        V Tbar, const FaceLine<V>& fl, V keep,
+                                                        V u_wall, V F[4])
+{
+    face_flux_tlbfs_wall<V>(L, Rc, Tbar, fl,
+                            [&](V& mn, V& mt, V rho) {
+                                mn = mn * keep;
+                                mt = vfma(keep, mt, rho * u_wall);
+                            },
+                            F);
 }
 
 // Parity of quantity k (0 drho, 1 u, 2 v, 3 T) about a wall of side s:

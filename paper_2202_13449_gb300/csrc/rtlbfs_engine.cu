@@ -142,21 +142,27 @@ int Engine::init()
     CK(cudaGetDevice(&dev));
     CK(cudaDeviceGetAttribute(&sms_, cudaDevAttrMultiProcessorCount, dev));
     CK(step_prepare(precision_));
-    for (int h : kTileHeights) {
-        if (!tile_height_ok(precision_, h)) continue;
-        CK(step_occupancy(precision_, h, kSchemeRTLBFS, &occ_tile_[h]));
-        if (occ_tile_[h] < 1) return fail(RTLBFS_ERR_CUDA, "step kernel does not fit on an SM");
+    for (int w = 0; w < 3; ++w) {
+        // FP32 blocks of width w run up to 2 / w to an SM (rebuild: wide_)
+        const int need = precision_ == RTLBFS_FP32 && w ? 2 / w : 1;
+        for (int h : kTileHeights) {
+            if (!tile_height_ok(precision_, h)) continue;
+            CK(step_occupancy(precision_, h, kSchemeRTLBFS, w, &occ_tile_[w][h]));
+            if (occ_tile_[w][h] < need) return fail(RTLBFS_ERR_CUDA, "step kernel does not fit on an SM");
+        }
+        CK(step_occupancy(precision_, kTileYDefault, kSchemeTLBFS, w, &occ_tlbfs_[w]));
+        if (occ_tlbfs_[w] < need) return fail(RTLBFS_ERR_CUDA, "TLBFS step kernel does not fit on an SM");
     }
-    CK(step_occupancy(precision_, kTileYDefault, kSchemeTLBFS, &occ_tlbfs_));
-    if (occ_tlbfs_ < 1) return fail(RTLBFS_ERR_CUDA, "TLBFS step kernel does not fit on an SM");
     CK(persist_prepare(precision_));
     for (int h : kTileHeights) {
         if (!tile_height_ok(precision_, h)) continue;
-        // the smaller of the two widths a height may run at
-        int wide = 0;
-        CK(persist_occupancy(precision_, kTileX, h, &wide));
-        CK(persist_occupancy(precision_, tile_width(precision_, h), h, &occ_persist_[h]));
-        occ_persist_[h] = std::min(occ_persist_[h], wide);
+        int wide1 = 0, wide2 = 0;
+        CK(persist_occupancy(precision_, kTileX, h, 0, &occ_persist_[h]));
+        CK(persist_occupancy(precision_, tile_width(precision_, h), h, 0, &occ_narrow_[h]));
+        CK(persist_occupancy(precision_, kTileX, h, 1, &wide1));
+        CK(persist_occupancy(precision_, kTileX, h, 2, &wide2));
+        if (precision_ == RTLBFS_FP32 && (wide1 < 2 || wide2 < 1))
+            return fail(RTLBFS_ERR_CUDA, "persistent kernel does not fit on an SM");
     }
     CK(march_prepare(precision_));
     CK(march_occupancy(precision_, &occ_march_));
@@ -632,58 +638,65 @@ int Engine::set_chunk_rows(int rows)
     return RTLBFS_OK;
 }
 
-// Tile height for the current set of cavities: the tiles of one launch run
-// about ceil(tiles / SMs) deep on the busiest SM, and a tile of height h
-// costs its faces and gradient ring plus a fixed share (loads, barriers,
-// the residual), in face-equivalents: 65 h + 32 + 0.25 * 34 (h + 2) + 300.
-// FP32 leaves out heights below 8: one or two warps a block pass through a
-// tile's phases too slowly even when every tile has an SM of its own (64^2:
-// 10.0 us per step at h = 2, 7.0 at 4, 6.6 at 8, 6.7 at 14).  FP64 is bound
-// by its narrow units, for which every warp instruction counts the same
-// however few lanes it serves: the cost is a tile's FP64 warp instructions
+// Tile height for the current set of cavities, by a model of the step time
+// (us, FP32) or of the FP64 work of the busiest SM, which gets n = ceil(tiles
+// / SMs) tiles.
+// FP32, measured: one tile per SM (four times the warps a block) 3.1 + 0.145
+// h, two (twice the warps) 3.9 + 0.24 h; beyond, full rounds of the resident
+// blocks at the per-tile times of a large mesh (2048^2), which favour tall
+// tiles for their smaller halo.
+// FP64 is bound by its narrow units, for which every warp instruction counts
+// the same however few lanes it serves: a tile's FP64 warp instructions
 // (rounds of faces 175, of gradients 32, of updates 170).
 int Engine::pick_tile_height(double* us) const
 {
     if (scheme_ == kSchemeTLBFS) return kTileYDefault;
     int best_h = kTileYDefault;
     double best = 1e300;
-    long long best_deep = 1;
     for (int h : kTileHeights) {
         if (!tile_height_ok(precision_, h)) continue;
-        if (precision_ == RTLBFS_FP32 && h < 8) continue;
         const int w = tile_width(precision_, h);
         long long tiles = 0;
         for (int s = 0; s < capacity_; ++s)
             if (slots_[s].active)
                 tiles += (long long)((slots_[s].nx + w - 1) / w) * ((slots_[s].ny + h - 1) / h);
-        const long long deep = (tiles + sms_ - 1) / std::max(sms_, 1);
-        const double tile_cost =
-            precision_ == RTLBFS_FP64 ? (h == 2 ? 900.0 : h == 4 ? 2654.0 : h == 8 ? 4862.0 : 9310.0)
-                                      : 65.0 * h + 32.0 + 0.25 * 34.0 * (h + 2) + 300.0;
-        const double cost = (double)deep * tile_cost;
+        const long long n = (tiles + sms_ - 1) / std::max(sms_, 1);
+        double cost;
+        if (precision_ == RTLBFS_FP64) {
+            cost = (double)n * (h == 2 ? 900.0 : h == 4 ? 2654.0 : h == 8 ? 4862.0 : 9310.0);
+        } else if (n <= 1) {
+            cost = 3.1 + 0.145 * h;
+        } else if (n == 2) {
+            cost = 3.9 + 0.24 * h;
+        } else {
+            const double tile_us = h == 2    ? 0.55
+                                   : h == 4  ? 1.06
+                                   : h == 8  ? 1.45
+                                   : h == 10 ? 1.70
+                                   : h == 12 ? 2.09
+                                   : h == 14 ? 2.17
+                                             : 2.47;
+            const long long occ = std::max(occ_tile_[0][h], 1);
+            cost = 2.0 + tile_us * (double)((n + occ - 1) / occ * occ);
+        }
         if (cost < best * (1.0 - 1e-9)) {
             best = cost;
             best_h = h;
-            best_deep = deep;
         }
     }
-    if (us) {
-        // FP32 step time: 14-row tiles (cost 1378) one deep take 6.7 us, two
-        // 8.4, three 10.5, four (a full SM) 10.9, then 2.65 us a tile
-        const double f = best / (1378.0 * (double)best_deep);
-        *us = std::max(4.7 + (0.3 + 1.6 * (double)best_deep) * f, 2.65 * (double)best_deep * f);
-    }
+    if (us) *us = best;
     return best_h;
 }
 
-// Rows per unit of the FP32 marching kernel: a warp passes H + 3.5 rows (the
-// chunk and its prologue) in about max(1.32, 1 + 0.105 w) us a row when w
-// warps share the SM (measured: 1.32 us at 4, 1.86 at 8, 2.2 at 12).  Units
-// beyond a full wave of 12 warps per SM run in further waves.
+// Rows per unit of the FP32 marching kernel: a warp passes H + 2.4 rows (the
+// chunk and its prologue) in about 0.74 + 0.13 w us a row when w warps share
+// the SM (measured: 1.25 us at 4, 1.75 at 7, 2.3 at 12), and a launch costs
+// 2.2 us more.  Units beyond a full wave of 12 warps per SM run in further
+// waves.
 int Engine::pick_march_rows(double* us) const
 {
     const long long slots = (long long)sms_ * std::max(occ_march_, 1);
-    auto row_us = [](double w) { return std::max(1.32, 1.0 + 0.105 * w); };
+    auto row_us = [](double w) { return std::max(1.2, 0.74 + 0.13 * w); };
     int best_h = 16, maxny = 1;
     double best = 1e300;
     for (int s = 0; s < capacity_; ++s)
@@ -697,14 +710,14 @@ int Engine::pick_march_rows(double* us) const
         const long long waves = units / slots, rest = units % slots;
         double t = (double)waves * row_us((double)occ_march_);
         if (rest) t += row_us((double)((rest + sms_ - 1) / sms_));
-        t *= H + 3.5;
+        t *= H + 2.4;
         if (t < best * (1.0 - 1e-9)) {
             best = t;
             best_h = H;
         }
         if (H >= maxny) break;
     }
-    if (us) *us = best + 3.5;
+    if (us) *us = best + 2.2;
     return best_h;
 }
 
@@ -712,9 +725,9 @@ int Engine::rebuild_tiles()
 {
     std::vector<int4> t;
     // A single cavity, unless a schedule was set: FP32 marches where that is modelled faster
-    // (from about 0.7 M cells: 1024^2 36.3, 4096^2 351 us per step
-    // against the tiles' 42 and 557; 512^2 18.2 against 10.9), FP64 takes tiles
-    // (64^2: 29 us against 269 in 16-row chunks, a serial chain of 20 rows).
+    // (from about 1 M cells: 1024^2 33.4, 2048^2 99.5 us per step
+    // against the tiles' 35.3 and 133; 700^2 20.4 against 18.8), FP64 takes tiles
+    // (64^2: 17 us against 269 in 16-row chunks, a serial chain of 20 rows).
     // A batch marches: its cavities come and go, and a kernel that followed
     // the mix would change a cavity's rounding on the way.
     if (auto_kernel_) {
@@ -732,12 +745,10 @@ int Engine::rebuild_tiles()
             gexec_ = nullptr;
         }
         tile_h_ = h;
-        // the persistent kernel takes no tile of one column: 32 columns where
-        // the narrower tile would leave one
         tile_w_ = tile_width(precision_, h);
         if (kernel_ == 2)
             for (int s = 0; s < capacity_; ++s)
-                if (slots_[s].active && slots_[s].nx % tile_w_ == 1) tile_w_ = kTileX;
+                if (slots_[s].active) tile_w_ = persist_width(slots_[s].nx, slots_[s].ny, h);
         for (int s = 0; s < capacity_; ++s) {
             Cavity& c = slots_[s];
             if (!c.active) continue;
@@ -838,6 +849,11 @@ int Engine::prepare_launch()
     }
     // persistent grid: every SM full, never more blocks than work units
     int want, march_cap = 0;
+    // FP32 tiles: more warps a block while the SMs get one tile, or two
+    const int wide = kernel_ == 0 || precision_ != RTLBFS_FP32 ? 0
+                     : ntiles_ <= sms_                        ? 2
+                     : ntiles_ <= 2 * sms_                    ? 1
+                                                              : 0;
     if (kernel_ == 2) {
         int rc = persist_check();
         if (rc) return rc;
@@ -850,7 +866,7 @@ int Engine::prepare_launch()
         }
         want = ntiles_;
     } else if (kernel_ == 1) {
-        const int occ = scheme_ == kSchemeTLBFS ? occ_tlbfs_ : occ_tile_[tile_h_];
+        const int occ = scheme_ == kSchemeTLBFS ? occ_tlbfs_[wide] : occ_tile_[wide][tile_h_];
         want = std::max(1, std::min(sms_ * occ, std::max(ntiles_, 1)));
     } else {
         const int wpb = (precision_ == RTLBFS_FP32 ? kMarch2Threads : kMarchThreads) / 32;
@@ -861,12 +877,13 @@ int Engine::prepare_launch()
         // short (1024^2 in 16-row units: 46.7 -> 37.9 us)
         march_cap = capacity_ == 1 && want < sms_ * occ_march_ ? (want + sms_ - 1) / sms_ : 0;
     }
-    if ((want != grid_ || march_cap != march_cap_) && gexec_) {
+    if ((want != grid_ || march_cap != march_cap_ || wide != wide_) && gexec_) {
         cudaGraphExecDestroy(gexec_);
         gexec_ = nullptr;
     }
     grid_ = want;
     march_cap_ = march_cap;
+    wide_ = wide;
     return RTLBFS_OK;
 }
 
@@ -1188,6 +1205,15 @@ int Engine::arm(int slot, long long nsteps, double tol)
     return RTLBFS_OK;
 }
 
+// Columns of the persistent kernel's tiles: tile_width where those leave no
+// tile of one column and all fit at once, else 32.
+int Engine::persist_width(int nx, int ny, int h) const
+{
+    const int w = tile_width(precision_, h);
+    const long long tiles = (long long)((nx + w - 1) / w) * ((ny + h - 1) / h);
+    return nx % w == 1 || tiles > (long long)sms_ * occ_narrow_[h] ? kTileX : w;
+}
+
 // The persistent tile kernel takes one RTLBFS cavity whose tiles are all
 // resident at once and at least two cells wide and high (a tile's 2-cell
 // halo then lies in the eight tiles around it).
@@ -1208,7 +1234,8 @@ int Engine::persist_check()
         return fail(RTLBFS_ERR_ARG, "the persistent kernel takes whole meshes, not row strips");
     if ((c.nx % tile_w_) == 1 || (c.ny % tile_h_) == 1)
         return fail(RTLBFS_ERR_ARG, "the persistent kernel needs tiles at least 2 cells wide");
-    if ((long long)ntiles_ > (long long)sms_ * occ_persist_[tile_h_])
+    if ((long long)ntiles_ >
+        (long long)sms_ * (tile_w_ == kTileX ? occ_persist_ : occ_narrow_)[tile_h_])
         return fail(RTLBFS_ERR_ARG, "the mesh has more tiles than fit on the GPU at once");
     persist_slot_ = slot;
     return RTLBFS_OK;
@@ -1227,7 +1254,7 @@ int Engine::launch_steps(long long launches)
             const int n = (int)std::min<long long>(left, kPersistChunk);
             CK(cudaMemsetAsync(d_tstep_, 0, sizeof(int) * ntiles_, stream_));
             CK(cudaMemsetAsync(d_pctl_, 0, sizeof(PersistCtl), stream_));
-            CK(launch_persist(precision_, tile_w_, tile_h_, ntiles_, stream_, &d_desc_[persist_slot_],
+            CK(launch_persist(precision_, tile_w_, tile_h_, wide_, ntiles_, stream_, &d_desc_[persist_slot_],
                               &d_ctl_[persist_slot_].h[0], d_tiles_ + c.first_tile, d_tstep_, d_pctl_,
                               n, withhold_));
             g_launches++;
@@ -1245,7 +1272,7 @@ int Engine::launch_steps(long long launches)
     long long left = launches;
     int par = 0;
     auto launch = [&](cudaStream_t st, int p) {
-        return kernel_ == 1 ? launch_step(precision_, tile_h_, scheme_, grid_, st, d_desc_, d_ctl_,
+        return kernel_ == 1 ? launch_step(precision_, tile_h_, scheme_, wide_, grid_, st, d_desc_, d_ctl_,
                                           d_tiles_, d_ntiles_, p)
                             : launch_march(precision_, grid_, march_cap_, st, d_desc_, d_ctl_,
                                            d_tiles_, d_ntiles_, p);
@@ -1325,10 +1352,10 @@ int Engine::autotune(int steps, int* kernel_out, int* rows_out, double* ms_out)
         for (int h : kTileHeights) {
             if (!tile_height_ok(precision_, h)) continue;
             const Cavity& c = slots_[aslot];
-            const int w = c.nx % tile_width(precision_, h) == 1 ? kTileX : tile_width(precision_, h);
+            const int w = persist_width(c.nx, c.ny, h);
             const long long tiles = (long long)((c.nx + w - 1) / w) * ((c.ny + h - 1) / h);
             if ((c.nx % kTileX) != 1 && (c.ny % h) != 1 &&
-                tiles <= (long long)sms_ * occ_persist_[h])
+                tiles <= (long long)sms_ * (w == kTileX ? occ_persist_ : occ_narrow_)[h])
                 cands.push_back({2, h});
         }
     if (scheme_ != kSchemeTLBFS) {

@@ -163,9 +163,12 @@ private:
     int capacity_;
     size_t rsize_;
     int sms_ = 0, grid_ = 0;
-    int occ_tile_[32] = {};  // resident tile blocks per SM, by tile height
-    int occ_tlbfs_ = 0;      // the same for the TLBFS tile kernel
-    int occ_persist_[32] = {};  // the same for the persistent tile kernel
+    int occ_tile_[3][32] = {};  // resident tile blocks per SM, by width of block and tile height
+    int occ_tlbfs_[3] = {};     // the same for the TLBFS tile kernel
+    int wide_ = 0;              // tile kernel, FP32: width of block (launch_step)
+    int occ_persist_[32] = {};  // the same for the persistent tile kernel, 32 columns wide
+    int occ_narrow_[32] = {};   // ... and tile_width wide
+    int persist_width(int nx, int ny, int h) const;
     int* d_tstep_ = nullptr;    // persistent kernel: last step of each tile
     int tstep_cap_ = 0;
     PersistCtl* d_pctl_ = nullptr;

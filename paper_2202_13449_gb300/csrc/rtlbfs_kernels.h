@@ -49,10 +49,12 @@ struct NuLines {
 // face stage, 0 RTLBFS, 1 TLBFS (tile height kTileYDefault only)
 constexpr int kSchemeRTLBFS = 0, kSchemeTLBFS = 1;
 cudaError_t step_prepare(int precision);
-cudaError_t step_occupancy(int precision, int tile_h, int scheme, int* blocks_per_sm);
+// wide (FP32): blocks of twice (1) or four times (2) the warps, for grids
+// that leave the SMs room
+cudaError_t step_occupancy(int precision, int tile_h, int scheme, int wide, int* blocks_per_sm);
 // par: parity of the launch within a chain of step launches (launch k of
 // a chain reads run header k & 1 and writes the other, see CavityRun)
-cudaError_t launch_step(int precision, int tile_h, int scheme, int grid, cudaStream_t s,
+cudaError_t launch_step(int precision, int tile_h, int scheme, int wide, int grid, cudaStream_t s,
                         const CavityDesc* descs, CavityRun* runs, const int4* tiles,
                         const int* ntiles, int par);
 cudaError_t march_prepare(int precision);
@@ -84,10 +86,10 @@ struct PersistCtl {
 // tile never reports its progress, so the waits of its neighbours run out.
 cudaError_t persist_prepare(int precision);
 // tile_w: tile_width, or kTileX where that would leave a tile of one column
-cudaError_t persist_occupancy(int precision, int tile_w, int tile_h, int* blocks_per_sm);
-cudaError_t launch_persist(int precision, int tile_w, int tile_h, int ntiles, cudaStream_t s,
-                           const CavityDesc* desc, CavityCtl* ctl, const int4* tiles, int* tstep,
-                           PersistCtl* pc, int nsteps, int withhold);
+cudaError_t persist_occupancy(int precision, int tile_w, int tile_h, int wide, int* blocks_per_sm);
+cudaError_t launch_persist(int precision, int tile_w, int tile_h, int wide, int ntiles,
+                           cudaStream_t s, const CavityDesc* desc, CavityCtl* ctl,
+                           const int4* tiles, int* tstep, PersistCtl* pc, int nsteps, int withhold);
 cudaError_t launch_nusselt(int precision, cudaStream_t s, const CavityDesc* descs,
                            const CavityRun* runs, int slot, const NuLines& ln, int which,
                            long long count, double scale, double* partial, int max_blocks,

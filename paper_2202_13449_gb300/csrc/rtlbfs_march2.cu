@@ -38,15 +38,13 @@
 
 #include "rtlbfs_dev.cuh"
 #include "rtlbfs_kernels.h"
+#include "rtlbfs_pair.cuh"
 
 namespace rtlbfs {
 
 namespace {
 
 using P = StoreQ;
-using Rec = Vec4<int>;
-
-__device__ __forceinline__ f2 splat(float v) { return {v, v}; }
 
 // Asynchronous global -> shared copy of a 16-byte record.
 __device__ __forceinline__ void copy_async(void* dst, const void* src)
@@ -61,92 +59,6 @@ __device__ __forceinline__ void copy_wait()
     asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-// two adjacent records at a 32-byte boundary in one access
-__device__ __forceinline__ void st2(Rec* p, const Rec& a, const Rec& b)
-{
-    asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "r"(a.x), "r"(a.y),
-                 "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w));
-}
-
-// A column's source on a line of n cells: the cell itself, the opposite
-// cell of a periodic line, or the cell that a ghost up to two beyond a wall
-// mirrors (m1, then m2: the sides to mirror across, -1: none).  Columns that
-// no stencil uses give false.
-__device__ __forceinline__ bool column_source(int c, int n, bool per, int& src, int& m1, int& m2)
-{
-    m1 = m2 = -1;
-    src = c;
-    if (c >= 0 && c < n) return true;
-    if (per) {
-        src = ((c % n) + n) % n;
-        return true;
-    }
-    if (c < -2 || c > n + 1) return false;
-    if (c < 0) {
-        m1 = kSideW;
-        src = -1 - c;
-        if (src >= n) {  // a line of one cell: the partner is itself a ghost
-            m2 = m1;
-            m1 = kSideE;
-            src = 2 * n - 1 - src;
-        }
-    } else {
-        m1 = kSideE;
-        src = 2 * n - 1 - c;
-        if (src < 0) {
-            m2 = m1;
-            m1 = kSideW;
-            src = -1 - src;
-        }
-    }
-    return true;
-}
-
-// Ghost values across wall `side` from the partner's working values (rho - 1,
-// u, v, T - Tref): rho even, velocity odd about the wall velocity (normal
-// component about 0), T odd about T_wall on a Dirichlet wall, even on an
-// adiabatic one.
-__device__ __forceinline__ void mirror_values2(const CavityDesc* d, int side, float Tref, float v[4])
-{
-    const float ut2 = 2.0f * P::bcU(d, side);
-    if (side == kSideW || side == kSideE) {
-        v[1] = -v[1];
-        v[2] = ut2 - v[2];
-    } else {
-        v[2] = -v[2];
-        v[1] = ut2 - v[1];
-    }
-    if (d->kind[side] == kDirichlet) v[3] = 2.0f * (P::Tw(d, side) - Tref) - v[3];
-}
-
-// Gradient of a ghost row across a south or north wall: even quantities
-// negate the normal part, odd ones the tangential part.
-__device__ __forceinline__ void mirror_grad_rows(int kind, f2 gx[4], f2 gy[4])
-{
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        if (wall_parity(kind, k) > 0) gy[k] = vtraits<f2>::neg(gy[k]);
-        else gx[k] = vtraits<f2>::neg(gx[k]);
-    }
-}
-
-// Working values (rho - 1, u, v, T - Tz) of two records.
-__device__ __forceinline__ void convert2(const Rec& a, const Rec& b, int qTz, f2 v[4])
-{
-    const f2 x[4] = {{(float)a.x, (float)b.x},
-                     {(float)a.y, (float)b.y},
-                     {(float)a.z, (float)b.z},
-                     {(float)(int)((unsigned)a.w - (unsigned)qTz),
-                      (float)(int)((unsigned)b.w - (unsigned)qTz)}};
-#pragma unroll
-    for (int k = 0; k < 4; ++k) v[k] = x[k] * splat(P::scale_f(k));
-}
-
-// Constants of a pair of faces.
-struct Line2 {
-    f2 h, cL, cR, m_nu_2h, m_chi_2h, m_tf15, m_tg15;
-};
-
 // What a warp keeps in shared memory; every lane reads back only what it
 // wrote or copied itself, so no synchronisation is needed.
 // line: the x-face constants, the same for every row.
@@ -158,51 +70,6 @@ struct WarpSmem {
     Rec row[kRing][2][32];
     f2 line[7][32];
 };
-
-// Fluxes of two faces with the same orientation from the cells on either
-// side (working values v, gradients along x and y in storage order): F =
-// (mass, x-, y-momentum, energy).  ISX: x-faces (normal u, tangential v).
-template <bool ISX, class W>
-__device__ __forceinline__ void faces2(const f2 vl[4], const f2 gxl[4], const f2 gyl[4],
-                                       const f2 vr[4], const f2 gxr[4], const f2 gyr[4], f2 Tz,
-                                       const Line2& ln, W wall, f2 F[4])
-{
-    constexpr int N = ISX ? 1 : 2, S = ISX ? 2 : 1;
-    constexpr int q[4] = {0, N, S, 3};
-    const f2* nl = ISX ? gxl : gyl;
-    const f2* tl = ISX ? gyl : gxl;
-    const f2* nr = ISX ? gxr : gyr;
-    const f2* tr = ISX ? gyr : gxr;
-    CellNT<f2> L, R;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        L.q[k] = vl[q[k]];
-        R.q[k] = vr[q[k]];
-        L.gn[k] = nl[q[k]];
-        R.gn[k] = nr[q[k]];
-        L.gt[k] = tl[q[k]];
-        R.gt[k] = tr[q[k]];
-    }
-    FaceLine<f2> fl;
-    fl.h = ln.h;
-    fl.cL = ln.cL;
-    fl.cR = ln.cR;
-    fl.m_nu_2h = ln.m_nu_2h;
-    fl.m_chi_2h = ln.m_chi_2h;
-    fl.m_tf15 = ln.m_tf15;
-    fl.m_tg15 = ln.m_tg15;
-    // temperatures relative to the left cell's (its own deviation is 0)
-    const f2 Tbar = Tz + L.q[3];
-    f2 A[4], Na[4], M[4], D[4], B[4], Sb[4], G[4];
-    R.q[3] = R.q[3] - L.q[3];
-    L.q[3] = splat(0.0f);
-    face_columns<f2>(L, R, fl, A, Na, M, D, B, Sb);
-    face_flux_wall<f2>(A, Na, M, D, B, Sb, Tbar, fl, wall, G);
-    F[0] = G[0];
-    F[N] = G[1];
-    F[S] = G[2];
-    F[3] = G[3];
-}
 
 __device__ __forceinline__ float up1(float v) { return __shfl_up_sync(0xffffffffu, v, 1); }
 __device__ __forceinline__ float dn1(float v) { return __shfl_down_sync(0xffffffffu, v, 1); }
@@ -276,28 +143,8 @@ march2_kernel(const CavityDesc* __restrict__ descs, CavityRun* __restrict__ runs
         const float Tz = P::val(qTz, 3);
         const f2 Tz2 = splat(Tz);
 
-        // raw records of row r (a ghost row: its partner's), ghost rules
-        // applied later in values()
-        auto row_source = [&](int r, int& rs, int& ym) -> bool {
-            ym = -1;
-            rs = r;
-            if ((r >= 0 && r < ny) || (r < 0 && hlo && r >= -2) || (r >= ny && hhi && r <= ny + 1))
-                return true;
-            if (yper) {
-                rs = ((r % ny) + ny) % ny;
-                return true;
-            }
-            if (r == -1) {
-                rs = 0;
-                ym = kSideS;
-                return true;
-            }
-            if (r == ny) {
-                rs = ny - 1;
-                ym = kSideN;
-                return true;
-            }
-            return false;
+        auto row = [&](int r, int& rs, int& ym) {
+            return row_source(r, ny, yper, hlo, hhi, rs, ym);
         };
         // the records this lane's columns take their values from (a column
         // that no stencil uses: any record)
@@ -310,27 +157,23 @@ march2_kernel(const CavityDesc* __restrict__ descs, CavityRun* __restrict__ runs
         auto fetch = [&](int r) {
             int rs, ym;
             if (r <= j1 + 1) {
-                if (!row_source(r, rs, ym)) rs = 0;
-                const Rec* row = fin + (long long)rs * pitch;
-                copy_async(&sm.row[r & (kRing - 1)][0][lane], row + sa);
-                copy_async(&sm.row[r & (kRing - 1)][1][lane], row + sb);
+                if (!row(r, rs, ym)) rs = 0;
+                const Rec* src = fin + (long long)rs * pitch;
+                copy_async(&sm.row[r & (kRing - 1)][0][lane], src + sa);
+                copy_async(&sm.row[r & (kRing - 1)][1][lane], src + sb);
             }
         };
         auto values = [&](int r, f2 v[4]) {
             convert2(sm.row[r & (kRing - 1)][0][lane], sm.row[r & (kRing - 1)][1][lane], qTz, v);
             int rs, ym;
-            const bool ok = row_source(r, rs, ym);
+            const bool ok = row(r, rs, ym);
             if (inside && ym < 0 && ok) return;  // warp-uniform
             auto ghost = [&](int c, float w[4]) {
                 int s, m1, m2;
-                if (!ok || !column_source(c, nx, xper, s, m1, m2)) {
-                    w[0] = w[1] = w[2] = w[3] = 0.0f;
-                    return;
-                }
-                if (ym >= 0) mirror_values2(dp, ym, Tz, w);
-                if (m1 >= 0) mirror_values2(dp, m1, Tz, w);
-                if (m2 >= 0) mirror_values2(dp, m2, Tz, w);
+                const bool used = column_source(c, nx, xper, s, m1, m2) && ok;
+                mirror_column(*dp, Tz, used, ym, m1, m2, w);
             };
+            // (the descriptor's wall values by address: once per ghost row or edge strip)
             float wa[4] = {v[0].x, v[1].x, v[2].x, v[3].x}, wb[4] = {v[0].y, v[1].y, v[2].y, v[3].y};
             ghost(ga, wa);
             ghost(ga + 1, wb);
@@ -351,10 +194,8 @@ march2_kernel(const CavityDesc* __restrict__ descs, CavityRun* __restrict__ runs
         // y-faces between rows jf - 1 (l) and jf (r)
         auto yfaces = [&](int jf, const FaceLine<float>& p, const f2 vl[4], const f2 gxl[4], const f2 gyl[4], const f2 vr[4],
                           const f2 gxr[4], const f2 gyr[4], f2 F[4]) {
-            const Line2 ly = {splat(p.h), splat(p.cL), splat(p.cR), splat(p.m_nu_2h),
-                              splat(p.m_chi_2h), splat(p.m_tf15), splat(p.m_tg15)};
             const int ws = (wall_s && jf == 0) ? kSideS : ((wall_n && jf == ny) ? kSideN : -1);
-            faces2<false>(vl, gxl, gyl, vr, gxr, gyr, Tz2, ly,
+            faces2<false, 0>(vl, gxl, gyl, vr, gxr, gyr, Tz2, splat_line(p),
                           [&](f2& mn, f2& mt, f2 rho) {
                               if (ws >= 0) {  // warp-uniform
                                   mn = splat(0.0f);
@@ -401,8 +242,7 @@ march2_kernel(const CavityDesc* __restrict__ descs, CavityRun* __restrict__ runs
             yfaces(j0, yl[min(max(j0, 0), ny)], vm, gxm, gym, v0, gx0, gy0, Fs);
         }
 
-        f2 s0 = splat(0.0f), s1 = s0, s2 = s0, s3 = s0;
-        bool bad = false;
+        PairSums acc;
 
         for (int j = j0; j < j1; ++j) {
             // this row's line constants, asked for before they are needed
@@ -413,15 +253,16 @@ march2_kernel(const CavityDesc* __restrict__ descs, CavityRun* __restrict__ runs
             f2 dF[4];
             {
                 f2 vl[4], gxl[4], gyl[4], Fx[4];
-                const Line2 lx = {sm.line[0][lane], sm.line[1][lane], sm.line[2][lane], sm.line[3][lane],
-                                  sm.line[4][lane], sm.line[5][lane], sm.line[6][lane]};
+                const FaceLine<f2> lx = {sm.line[0][lane], sm.line[1][lane], sm.line[2][lane],
+                                         sm.line[3][lane], sm.line[4][lane], sm.line[5][lane],
+                                         sm.line[6][lane], splat(0.0f)};
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
                     vl[k] = {up1(v0[k].y), v0[k].x};
                     gxl[k] = {up1(gx0[k].y), gx0[k].x};
                     gyl[k] = {up1(gy0[k].y), gy0[k].x};
                 }
-                faces2<true>(vl, gxl, gyl, v0, gx0, gy0, Tz2, lx,
+                faces2<true, 0>(vl, gxl, gyl, v0, gx0, gy0, Tz2, lx,
                              [&](f2& mn, f2& mt, f2 rho) {
                                  if (xwall) {  // warp-uniform
                                      const bool wa = ga == 0 || ga == nx, wb = ga + 1 == nx;
@@ -469,42 +310,8 @@ march2_kernel(const CavityDesc* __restrict__ descs, CavityRun* __restrict__ runs
                 f2 div[4];
 #pragma unroll
                 for (int k = 0; k < 4; ++k) div[k] = vfma(dtx, dF[k], splat(dty) * (Fn[k] - Fs[k]));
-                const f2 dr = v0[0], u = v0[1], v = v0[2], T = Tz2 + v0[3];
-                const f2 rho = splat(1.0f) + dr;
-                const f2 src_x = rho * splat(sfx);
-                const f2 src_y = rho * vfma(splat(sbg), T - splat(Tr), splat(sfy));
-                const f2 inv = vtraits<f2>::rcp(rho - div[0]);
-                const f2 du = (vfma(u, div[0], src_x) - div[1]) * inv;
-                const f2 dv = (vfma(v, div[0], src_y) - div[2]) * inv;
-                const f2 dT = (T * div[0] - div[3]) * inv;
-                const f2 dr1 = dr - div[0], u1 = u + du, v1n = v + dv, T1 = T + dT;
-                Rec* const outp = fout + (size_t)j * pitch + ga;
-                const Rec qa = sm.row[j & (kRing - 1)][0][lane], qb = sm.row[j & (kRing - 1)][1][lane];
-                const Rec oa = {P::add(qa.x, -div[0].x, 0), P::add(qa.y, du.x, 1),
-                                P::add(qa.z, dv.x, 2), P::add(qa.w, dT.x, 3)};
-                const Rec ob = {P::add(qb.x, -div[0].y, 0), P::add(qb.y, du.y, 1),
-                                P::add(qb.z, dv.y, 2), P::add(qb.w, dT.y, 3)};
-                const bool ba = !(P::in_range(dr1.x, 0) && P::in_range(u1.x, 1) &&
-                                  P::in_range(v1n.x, 2) && P::in_range(T1.x, 3));
-                const bool bb = !(P::in_range(dr1.y, 0) && P::in_range(u1.y, 1) &&
-                                  P::in_range(v1n.y, 2) && P::in_range(T1.y, 3));
-                const f2 q0 = vfma(u, u, v * v), q1 = vfma(u1, u1, v1n * v1n);
-                const f2 den = f2{P::fsqrt(q0.x), P::fsqrt(q0.y)} + f2{P::fsqrt(q1.x), P::fsqrt(q1.y)};
-                const f2 num = vfma(du, u + u1, dv * (v + v1n));
-                f2 dm = {den.x > 0.0f ? num.x * P::rcp(den.x) : 0.0f,
-                         den.y > 0.0f ? num.y * P::rcp(den.y) : 0.0f};
-                f2 e1 = q1, e2 = dT, e3 = T1;
-                bad = bad || ba || (bb && upd_b);
-                if (upd_b) {
-                    st2(outp, oa, ob);
-                } else {  // the last column of an odd line: cell b is not a cell
-                    *outp = oa;
-                    dm.y = e1.y = e2.y = e3.y = 0.0f;
-                }
-                s0 = vfma(dm, dm, s0);
-                s1 = s1 + e1;
-                s2 = vfma(e2, e2, s2);
-                s3 = vfma(e3, e3, s3);
+                update2(v0, Tz, div, sfx, sfy, sbg, Tr, sm.row[j & (kRing - 1)][0][lane],
+                        sm.row[j & (kRing - 1)][1][lane], upd_b, fout + (size_t)j * pitch + ga, acc);
             }
             // roll the window
 #pragma unroll
@@ -516,8 +323,7 @@ march2_kernel(const CavityDesc* __restrict__ descs, CavityRun* __restrict__ runs
                 gy0[k] = gy1[k];
             }
         }
-        float a0 = bad ? NAN : s0.x + s0.y, a1 = s1.x + s1.y, a2 = s2.x + s2.y, a3 = s3.x + s3.y;
-        const float sum = warp_sum4(a0, a1, a2, a3);
+        const float sum = warp_total(acc);
         // the step's residual sums; the next launch tests them
         if ((lane & 7) == 0) atomicAdd(&run->acc[slot3][lane >> 3], (double)sum);
         __syncwarp();

@@ -82,7 +82,7 @@ __device__ bool warp_wait(const int* p, int v, const int* q, int* stalled)
 }  // namespace
 
 template <class P, int TX, int TY, int NT>
-__global__ void __launch_bounds__(NT, MinBlocks<P, NT>::value)
+__global__ void __launch_bounds__(NT, MinBlocks<P, TX, TY, NT>::value)
 persist_kernel(const CavityDesc* __restrict__ dp, CavityCtl* __restrict__ ctl,
                const int4* __restrict__ tiles, int* __restrict__ tstep,
                PersistCtl* __restrict__ pc, int nsteps, int withhold)
@@ -149,9 +149,9 @@ persist_kernel(const CavityDesc* __restrict__ dp, CavityCtl* __restrict__ ctl,
         __syncthreads();
         if (sm.last != 1) break;  // uniform: stopped, or stalled
         const int rb = c0 ^ ((k - 1) & 1);  // buffer with the state after step k - 1
-        run_tile<P, TX, TY, NT, 0, true>(sm, &sm.desc, i0, j0,
+        run_tile<P, TX, TY, NT, 0, true>(sm, i0, j0,
                                          static_cast<const Vec4<S>*>(dp->f[rb][0]),
-                                         static_cast<Vec4<S>*>(dp->f[rb ^ 1][0]), true);
+                                         static_cast<Vec4<S>*>(dp->f[rb ^ 1][0]));
         __syncthreads();
         double* acc = pc->acc[k % 3];
         tile_sums(sm, acc);  // threads 0-3
@@ -188,9 +188,9 @@ persist_kernel(const CavityDesc* __restrict__ dp, CavityCtl* __restrict__ ctl,
     }
 }
 
-template <class P, int TY, int TX = kTileX>
+template <class P, int TY, int WIDE = 0, int TX = kTileX>
 struct PersistKernel {
-    static constexpr int NT = TileThreads<P, TX, TY>::value;
+    static constexpr int NT = TileThreads<P, TX, TY, WIDE>::value;
     static constexpr size_t smem = sizeof(TileSmem<P, TX, TY, NT>);
     static constexpr auto fn = persist_kernel<P, TX, TY, NT>;
     static cudaError_t prepare()
@@ -222,31 +222,38 @@ struct PersistKernel {
     }
 };
 
+template <int WIDE, class Op>
+static cudaError_t with_persist_kernel_q(int tile_h, Op op)
+{
+    switch (tile_h) {
+    case 16: return op(PersistKernel<StoreQ, 16, WIDE>());
+    case 14: return op(PersistKernel<StoreQ, 14, WIDE>());
+    case 12: return op(PersistKernel<StoreQ, 12, WIDE>());
+    case 10: return op(PersistKernel<StoreQ, 10, WIDE>());
+    case 8: return op(PersistKernel<StoreQ, 8, WIDE>());
+    case 4: return op(PersistKernel<StoreQ, 4, WIDE>());
+    case 2: return op(PersistKernel<StoreQ, 2, WIDE>());
+    default: return cudaErrorInvalidValue;
+    }
+}
+
 template <class Op>
-static cudaError_t with_persist_kernel(int precision, int tile_w, int tile_h, Op op)
+static cudaError_t with_persist_kernel(int precision, int tile_w, int tile_h, int wide, Op op)
 {
     if (tile_w != kTileX) {
         if (precision == 0 && tile_h == 2 && tile_w == tile_width(0, 2))
-            return op(PersistKernel<StoreD, 2, tile_width(0, 2)>());
+            return op(PersistKernel<StoreD, 2, 0, tile_width(0, 2)>());
         return cudaErrorInvalidValue;
     }
-    if (precision == 0) {
-        switch (tile_h) {
-        case 16: return op(PersistKernel<StoreD, 16>());
-        case 8: return op(PersistKernel<StoreD, 8>());
-        case 4: return op(PersistKernel<StoreD, 4>());
-        case 2: return op(PersistKernel<StoreD, 2>());
-        default: return cudaErrorInvalidValue;
-        }
-    }
+    if (precision != 0)
+        return wide == 2   ? with_persist_kernel_q<2>(tile_h, op)
+               : wide == 1 ? with_persist_kernel_q<1>(tile_h, op)
+                           : with_persist_kernel_q<0>(tile_h, op);
     switch (tile_h) {
-    case 16: return op(PersistKernel<StoreQ, 16>());
-    case 14: return op(PersistKernel<StoreQ, 14>());
-    case 12: return op(PersistKernel<StoreQ, 12>());
-    case 10: return op(PersistKernel<StoreQ, 10>());
-    case 8: return op(PersistKernel<StoreQ, 8>());
-    case 4: return op(PersistKernel<StoreQ, 4>());
-    case 2: return op(PersistKernel<StoreQ, 2>());
+    case 16: return op(PersistKernel<StoreD, 16>());
+    case 8: return op(PersistKernel<StoreD, 8>());
+    case 4: return op(PersistKernel<StoreD, 4>());
+    case 2: return op(PersistKernel<StoreD, 2>());
     default: return cudaErrorInvalidValue;
     }
 }
@@ -255,25 +262,27 @@ cudaError_t persist_prepare(int precision)
 {
     for (int h : kTileHeights) {
         if (!tile_height_ok(precision, h)) continue;
-        for (int w : {kTileX, tile_width(precision, h)}) {
-            cudaError_t e = with_persist_kernel(precision, w, h, [](auto k) { return k.prepare(); });
-            if (e != cudaSuccess) return e;
-        }
+        for (int w : {kTileX, tile_width(precision, h)})
+            for (int wide : {0, 1, 2}) {
+                cudaError_t e =
+                    with_persist_kernel(precision, w, h, wide, [](auto k) { return k.prepare(); });
+                if (e != cudaSuccess) return e;
+            }
     }
     return cudaSuccess;
 }
 
-cudaError_t persist_occupancy(int precision, int tile_w, int tile_h, int* blocks_per_sm)
+cudaError_t persist_occupancy(int precision, int tile_w, int tile_h, int wide, int* blocks_per_sm)
 {
-    return with_persist_kernel(precision, tile_w, tile_h,
+    return with_persist_kernel(precision, tile_w, tile_h, wide,
                                [&](auto k) { return k.occupancy(blocks_per_sm); });
 }
 
-cudaError_t launch_persist(int precision, int tile_w, int tile_h, int ntiles, cudaStream_t s,
-                           const CavityDesc* desc, CavityCtl* ctl, const int4* tiles, int* tstep,
-                           PersistCtl* pc, int nsteps, int withhold)
+cudaError_t launch_persist(int precision, int tile_w, int tile_h, int wide, int ntiles,
+                           cudaStream_t s, const CavityDesc* desc, CavityCtl* ctl,
+                           const int4* tiles, int* tstep, PersistCtl* pc, int nsteps, int withhold)
 {
-    return with_persist_kernel(precision, tile_w, tile_h, [&](auto k) {
+    return with_persist_kernel(precision, tile_w, tile_h, wide, [&](auto k) {
         return k.launch(ntiles, s, desc, ctl, tiles, tstep, pc, nsteps, withhold);
     });
 }

@@ -33,7 +33,7 @@
 namespace rtlbfs {
 
 template <class P, int TX, int TY, int NT, int SCHEME>
-__global__ void __launch_bounds__(NT, MinBlocks<P, NT>::value)
+__global__ void __launch_bounds__(NT, MinBlocks<P, TX, TY, NT>::value)
 step_kernel(const CavityDesc* __restrict__ descs, CavityRun* __restrict__ runs,
             const int4* __restrict__ tiles, const int* __restrict__ ntiles_ptr, int par)
 {
@@ -51,32 +51,31 @@ step_kernel(const CavityDesc* __restrict__ descs, CavityRun* __restrict__ runs,
     }
     chain_sync();
 
+    int planned = -1;  // the cavity whose plan is in shared memory
     for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
         const int4 tile = tiles[t];
         const int slot = tile.x, i0 = tile.y, j0 = tile.z;
         CavityRun* run = &runs[slot];
+        if (t != (int)blockIdx.x) stage_tile(sm, &descs[slot], i0, j0);
         // the stop test of the cavity's previous step (one thread; its first
         // tile also publishes the header for the next launch)
-        if (tid == 0) {
+        if (tid == 0 && slot != planned) {
             const CavityCtl d = run_head(run, par);
             if (t == descs[slot].tile_begin) run_publish(run, par, d);
             sm.plan[0] = d.done;
             sm.plan[1] = d.cur;
             sm.plan[2] = (int)(d.steps % 3);
         }
-        __syncthreads();  // the plan (and, on the first tile, the staged descriptor and lines)
+        planned = slot;
+        __syncthreads();  // the plan, the staged descriptor and lines
         const int done = sm.plan[0], cur = sm.plan[1], slot3 = sm.plan[2];
         if (done) {  // uniform across the block
             __syncthreads();  // everyone has read the plan before it is rewritten
             continue;
         }
-        // the first tile uses what was staged; later tiles (batches) read
-        // their descriptor in place and load their lines beside the state
-        const bool first = t == (int)blockIdx.x;
-        const CavityDesc* dp = first ? &sm.desc : &descs[slot];
-        run_tile<P, TX, TY, NT, SCHEME, false>(sm, dp, i0, j0,
-                                               static_cast<const Vec4<S>*>(dp->f[cur][0]),
-                                               static_cast<Vec4<S>*>(dp->f[cur ^ 1][0]), first);
+        run_tile<P, TX, TY, NT, SCHEME, false>(sm, i0, j0,
+                                               static_cast<const Vec4<S>*>(sm.desc.f[cur][0]),
+                                               static_cast<Vec4<S>*>(sm.desc.f[cur ^ 1][0]));
         __syncthreads();
         tile_sums(sm, run->acc[slot3]);  // the next launch tests them
         __syncthreads();
@@ -326,10 +325,10 @@ __global__ void arm_kernel(CavityRun* runs, const int* __restrict__ slot_list, i
 // ---------------------------------------------------------------------------
 // host-side launchers
 // ---------------------------------------------------------------------------
-template <class P, int TY, int SCHEME = 0>
+template <class P, int TY, int SCHEME = 0, int WIDE = 0>
 struct TileKernel {
     static constexpr int TX = tile_width(sizeof(typename P::R) == 8 ? 0 : 1, TY);
-    static constexpr int NT = TileThreads<P, TX, TY>::value;
+    static constexpr int NT = TileThreads<P, TX, TY, WIDE>::value;
     static constexpr size_t smem = sizeof(TileSmem<P, TX, TY, NT>);
     static constexpr auto fn = step_kernel<P, TX, TY, NT, SCHEME>;
     static cudaError_t prepare()
@@ -352,59 +351,77 @@ struct TileKernel {
     }
 };
 
-// Call op on the compiled tile kernel of (precision, tile_h, scheme); the
-// TLBFS face stage is compiled for the default tile height.
-template <class Op>
-static cudaError_t with_tile_kernel(int precision, int tile_h, int scheme, Op op)
+// Call op on the compiled tile kernel of (precision, tile_h, scheme, wide);
+// the TLBFS face stage is compiled for the default tile height, wide blocks
+// for FP32.
+template <int WIDE, class Op>
+static cudaError_t with_tile_kernel_q(int tile_h, int scheme, Op op)
 {
     if (scheme == 1) {
         if (tile_h != kTileYDefault) return cudaErrorInvalidValue;
-        if (precision == 0) return op(TileKernel<StoreD, kTileYDefault, 1>());
-        return op(TileKernel<StoreQ, kTileYDefault, 1>());
-    }
-    if (scheme != 0) return cudaErrorInvalidValue;
-    if (precision == 0) {
-        switch (tile_h) {
-        case 16: return op(TileKernel<StoreD, 16>());
-        case 8: return op(TileKernel<StoreD, 8>());
-        case 4: return op(TileKernel<StoreD, 4>());
-        case 2: return op(TileKernel<StoreD, 2>());
-        default: return cudaErrorInvalidValue;
-        }
+        return op(TileKernel<StoreQ, kTileYDefault, 1, WIDE>());
     }
     switch (tile_h) {
-    case 16: return op(TileKernel<StoreQ, 16>());
-    case 14: return op(TileKernel<StoreQ, 14>());
-    case 12: return op(TileKernel<StoreQ, 12>());
-    case 10: return op(TileKernel<StoreQ, 10>());
-    case 8: return op(TileKernel<StoreQ, 8>());
-    case 4: return op(TileKernel<StoreQ, 4>());
-    case 2: return op(TileKernel<StoreQ, 2>());
+    case 16: return op(TileKernel<StoreQ, 16, 0, WIDE>());
+    case 14: return op(TileKernel<StoreQ, 14, 0, WIDE>());
+    case 12: return op(TileKernel<StoreQ, 12, 0, WIDE>());
+    case 10: return op(TileKernel<StoreQ, 10, 0, WIDE>());
+    case 8: return op(TileKernel<StoreQ, 8, 0, WIDE>());
+    case 4: return op(TileKernel<StoreQ, 4, 0, WIDE>());
+    case 2: return op(TileKernel<StoreQ, 2, 0, WIDE>());
+    default: return cudaErrorInvalidValue;
+    }
+}
+
+template <class Op>
+static cudaError_t with_tile_kernel(int precision, int tile_h, int scheme, int wide, Op op)
+{
+    if (scheme != 0 && scheme != 1) return cudaErrorInvalidValue;
+    if (precision != 0)
+        return wide == 2   ? with_tile_kernel_q<2>(tile_h, scheme, op)
+               : wide == 1 ? with_tile_kernel_q<1>(tile_h, scheme, op)
+                           : with_tile_kernel_q<0>(tile_h, scheme, op);
+    if (scheme == 1) {
+        if (tile_h != kTileYDefault) return cudaErrorInvalidValue;
+        return op(TileKernel<StoreD, kTileYDefault, 1>());
+    }
+    switch (tile_h) {
+    case 16: return op(TileKernel<StoreD, 16>());
+    case 8: return op(TileKernel<StoreD, 8>());
+    case 4: return op(TileKernel<StoreD, 4>());
+    case 2: return op(TileKernel<StoreD, 2>());
     default: return cudaErrorInvalidValue;
     }
 }
 
 cudaError_t step_prepare(int precision)
 {
-    for (int h : kTileHeights) {
-        if (!tile_height_ok(precision, h)) continue;
-        cudaError_t e = with_tile_kernel(precision, h, 0, [](auto k) { return k.prepare(); });
+    for (int wide = 0; wide < 3; ++wide) {
+        for (int h : kTileHeights) {
+            if (!tile_height_ok(precision, h)) continue;
+            cudaError_t e =
+                with_tile_kernel(precision, h, 0, wide, [](auto k) { return k.prepare(); });
+            if (e != cudaSuccess) return e;
+        }
+        cudaError_t e = with_tile_kernel(precision, kTileYDefault, 1, wide,
+                                         [](auto k) { return k.prepare(); });
         if (e != cudaSuccess) return e;
+        if (precision == 0) break;
     }
-    return with_tile_kernel(precision, kTileYDefault, 1, [](auto k) { return k.prepare(); });
+    return cudaSuccess;
 }
 
-cudaError_t step_occupancy(int precision, int tile_h, int scheme, int* blocks_per_sm)
+cudaError_t step_occupancy(int precision, int tile_h, int scheme, int wide, int* blocks_per_sm)
 {
-    return with_tile_kernel(precision, tile_h, scheme,
+    return with_tile_kernel(precision, tile_h, scheme, wide,
                             [&](auto k) { return k.occupancy(blocks_per_sm); });
 }
 
-cudaError_t launch_step(int precision, int tile_h, int scheme, int grid, cudaStream_t s,
+cudaError_t launch_step(int precision, int tile_h, int scheme, int wide, int grid, cudaStream_t s,
                         const CavityDesc* descs, CavityRun* runs, const int4* tiles,
                         const int* ntiles, int par)
 {
-    return with_tile_kernel(precision, tile_h, scheme, [&](auto k) {
+    return with_tile_kernel(precision, tile_h, scheme, wide, [&](auto k) {
         return k.launch(grid, s, descs, runs, tiles, ntiles, par);
     });
 }

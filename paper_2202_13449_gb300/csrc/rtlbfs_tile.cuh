@@ -17,7 +17,6 @@ namespace rtlbfs {
 
 template <class P, int TX, int TY, int NT>
 struct TileSmem {
-    using S = typename P::S;
     using R = typename P::R;
     static constexpr int BX = TX + 4, BY = TY + 4;  // tile + 2-cell halo
     static constexpr int GX = TX + 2, GY = TY + 2;  // gradient ring
@@ -28,12 +27,6 @@ struct TileSmem {
     Vec4<R> gy[GY][GX];
     Vec4<R> fx[TY][TX + 1];
     Vec4<R> fy[TY + 1][TX];
-    // the stored records of the tile's own cells, as loaded: the update
-    // adds its increments to them instead of reading the state again.  Only
-    // where the 16-byte records leave room for four resident blocks per SM
-    // (FP32 tiles up to 14 rows); elsewhere the update re-reads them (L2).
-    static constexpr bool kRaw = sizeof(S) == 4 && TY <= 14;
-    Vec4<S> raw[kRaw ? TY : 1][kRaw ? TX : 1];
     FaceLine<R> xl[TX + 1];
     FaceLine<R> yl[TY + 1];
     CellLine<R> xc[BX];
@@ -186,16 +179,6 @@ __device__ __forceinline__ void gg_gradient_r(const Vec4<R>& p, const Vec4<R>& e
     gy.w = (n.w - p.w) * iyn + (p.w - s.w) * iys;
 }
 
-// The same in FP32, two components per packed FP32x2 instruction.
-__device__ __forceinline__ void gg_gradient_r(const Vec4<float>& p, const Vec4<float>& e,
-                                              const Vec4<float>& w, const Vec4<float>& n,
-                                              const Vec4<float>& s, float ixe, float ixw,
-                                              float iyn, float iys, Vec4<float>& gx,
-                                              Vec4<float>& gy)
-{
-    gg_gradient_f32(p, e, w, n, s, ixe, ixw, iyn, iys, gx, gy);
-}
-
 template <typename R>
 __device__ __forceinline__ R warp_sum(R v)
 {
@@ -223,17 +206,6 @@ __device__ __forceinline__ void face_cells(bool isx, const Vec4<R>& vl, const Ve
         Rr = {{vr.x, vr.z, vr.y, tR}, {gyr.x, gyr.z, gyr.y, gyr.w}, {gxr.x, gxr.z, gxr.y, gxr.w}};
     }
 }
-
-// Resident blocks per SM to compile for: FP32 aims at 64 registers a thread
-// (the tile buffers then bound occupancy); FP64 takes what it needs.
-template <class P, int NT>
-struct MinBlocks {
-    static constexpr int value = 1;
-};
-template <int NT>
-struct MinBlocks<StoreQ, NT> {
-    static constexpr int value = 65536 / (NT * 64);
-};
 
 // The state record at p: through L2 only (LDCG, for a kernel whose blocks
 // read what other blocks of the same launch wrote; L1 is not coherent) or
@@ -278,7 +250,7 @@ __device__ __forceinline__ void stage_lines(TileSmem<P, TX, TY, NT>& sm, const C
 // descriptor (sm.desc) and the mesh lines of the tile and its halo.  Kernels
 // call it before they wait for the previous step, so these loads overlap
 // that step's tail instead of heading this step's chain of dependent loads;
-// a barrier must separate it from tile_step (called with lines_staged).
+// a barrier must separate it from run_tile.
 template <class P, int TX, int TY, int NT>
 __device__ __forceinline__ void stage_tile(TileSmem<P, TX, TY, NT>& sm, const CavityDesc* gdp,
                                            int i0, int j0)
@@ -305,12 +277,10 @@ __device__ __forceinline__ void tile_sums(const TileSmem<P, TX, TY, NT>& sm, dou
     add_sums(sm.red, FlatTile<P, TX, TY>::value ? 1 : NT / 32, acc);
 }
 
-// One tile of one time step on cavity *dp, tile origin (i0, j0): phases 1-4
-// below read the state from fin and write the new state to fout; the
-// tile's four residual sums are left in sm.red (a row per warp) for the
-// caller to add (tile_sums) after a barrier.  lines_staged: stage_tile has put the
-// tile's mesh lines in shared memory (dp may then point at its copy of the
-// descriptor); otherwise phase 1 loads them beside the state.
+// One tile of one time step, tile origin (i0, j0), on the cavity and mesh
+// lines that stage_tile has put in shared memory: phases 1-4 below read the
+// state from fin and write the new state to fout; the tile's four residual
+// sums are left in sm.red (a row per warp) for tile_sums after a barrier.
 //
 // Work of a thread.  The tile's TX x TY cells are split into CPT = TX*TY/NT
 // cells per thread at fixed places: thread (c, r) = (tid % CW, tid / CW),
@@ -324,12 +294,11 @@ __device__ __forceinline__ void tile_sums(const TileSmem<P, TX, TY, NT>& sm, dou
 // no warp computes two faces more than the others.  With CW = 16 or 32
 // lanes of a warp read consecutive records: no bank conflicts.
 template <class P, int TX, int TY, int NT, int SCHEME, bool LDCG>
-__device__ __forceinline__ void tile_step(TileSmem<P, TX, TY, NT>& sm, const CavityDesc* dp,
-                                          int i0, int j0,
+__device__ __forceinline__ void tile_step(TileSmem<P, TX, TY, NT>& sm, int i0, int j0,
                                           const Vec4<typename P::S>* __restrict__ fin,
-                                          Vec4<typename P::S>* __restrict__ fout,
-                                          bool lines_staged)
+                                          Vec4<typename P::S>* __restrict__ fout)
 {
+    const CavityDesc* const dp = &sm.desc;
     using Sm = TileSmem<P, TX, TY, NT>;
     using S = typename P::S;
     using R = typename P::R;
@@ -337,9 +306,6 @@ __device__ __forceinline__ void tile_step(TileSmem<P, TX, TY, NT>& sm, const Cav
     constexpr int CPT = TX * TY / NT;
     constexpr int CW = TX / CPT;
     static_assert(CPT * NT == TX * TY && CW * CPT == TX && CW * TY == NT, "thread layout");
-    // the gradient and face loops unrolled where that stays within the
-    // register budget of four resident blocks (FP32 tiles of 4+ rows)
-    constexpr int UNROLL = (sizeof(R) == 4 && TY >= 4) ? 8 : 1;
     const int tid = threadIdx.x;
     const int tc = tid % CW, tr = tid / CW;
     const int nx = dp->nx, ny = dp->ny, pitch = dp->pitch;
@@ -354,8 +320,7 @@ __device__ __forceinline__ void tile_step(TileSmem<P, TX, TY, NT>& sm, const Cav
     // ghost resolution, no mirror rules, no wall faces (block-uniform).
     const bool interior = i0 >= 2 && j0 >= 2 && i0 + TX + 2 <= nx && j0 + TY + 2 <= ny;
 
-    // ---- 1. mesh lines (unless staged) and the haloed tile -------------
-    if (!lines_staged) stage_lines(sm, dp, i0, j0);
+    // ---- 1. the haloed tile ---------------------------------------------
     {
         // box positions (column, row) of load k: own cells, then the ring
         // (the two rows below, the two above, two columns each side)
@@ -402,10 +367,6 @@ __device__ __forceinline__ void tile_step(TileSmem<P, TX, TY, NT>& sm, const Cav
                 if (ok[k]) v[k] = ld_state<LDCG>(&fin[(long long)sj * pitch + si]);
             }
         }
-        if constexpr (Sm::kRaw) {
-#pragma unroll
-            for (int k = 0; k < CPT; ++k) sm.raw[tr][tc + k * CW] = v[k];
-        }
 #pragma unroll
         for (int k = 0; k < NL; ++k) {
             int bc = 0, br = 0;
@@ -425,7 +386,7 @@ __device__ __forceinline__ void tile_step(TileSmem<P, TX, TY, NT>& sm, const Cav
     {
         constexpr int NGR = GX * GY - TX * TY;
         constexpr int GQ = CPT + (NGR + NT - 1) / NT;
-#pragma unroll(UNROLL)
+#pragma unroll 1
         for (int k = 0; k < GQ; ++k) {
             int gc, gr;
             if (k < CPT) {
@@ -493,16 +454,6 @@ __device__ __forceinline__ void tile_step(TileSmem<P, TX, TY, NT>& sm, const Cav
             R F[4];
             if constexpr (SCHEME == 1) {
                 face_flux_tlbfs<R>(L, Rr, Tbar, fl, wside >= 0 ? R(0) : R(1), uw, F);
-            } else if constexpr (sizeof(R) == 4) {
-                // FP32: the column stage in packed pairs of the storage order
-                const Vec4<R> gl = isx ? sm.gx[lr - 1][lc - 1] : sm.gy[lr - 1][lc - 1];
-                const Vec4<R> tl = isx ? sm.gy[lr - 1][lc - 1] : sm.gx[lr - 1][lc - 1];
-                const Vec4<R> gr = isx ? sm.gx[rr - 1][rc - 1] : sm.gy[rr - 1][rc - 1];
-                const Vec4<R> tr = isx ? sm.gy[rr - 1][rc - 1] : sm.gx[rr - 1][rc - 1];
-                R A[4], Na[4], M[4], D[4], B[4], Sb[4];
-                face_columns_f32<isx>(sm.val[lr][lc], sm.val[rr][rc], gl, tl, gr, tr, fl, A, Na, M,
-                                      D, B, Sb);
-                face_flux_columns<R>(A, Na, M, D, B, Sb, Tbar, fl, wside >= 0 ? R(0) : R(1), uw, F);
             } else {
                 face_flux<R>(L, Rr, Tbar, fl, wside >= 0 ? R(0) : R(1), uw, F);
             }
@@ -521,7 +472,7 @@ __device__ __forceinline__ void tile_step(TileSmem<P, TX, TY, NT>& sm, const Cav
         // warps, and no warp computes two faces more than the others
         constexpr int EW = (TY + 31) / 32 * 32;
         constexpr int YOFF = EW + TX <= TQ * NT ? EW : TY;
-#pragma unroll(UNROLL)
+#pragma unroll 1
         for (int k = 0; k < CPT + TQ; ++k) {
             int fc = tc + k * CW, fr = tr;
             if (k >= CPT) {
@@ -532,7 +483,7 @@ __device__ __forceinline__ void tile_step(TileSmem<P, TX, TY, NT>& sm, const Cav
             }
             face(XF(), fc, fr);
         }
-#pragma unroll(UNROLL)
+#pragma unroll 1
         for (int k = 0; k < CPT + TQ; ++k) {
             int fc = tc + k * CW, fr = tr;
             if (k >= CPT) {
@@ -560,9 +511,7 @@ __device__ __forceinline__ void tile_step(TileSmem<P, TX, TY, NT>& sm, const Cav
             const int gi = i0 + cc, gj = j0 + tr;
             if (gi >= nx || gj >= ny) continue;
             const size_t o = (size_t)gj * pitch + gi;
-            Vec4<S> q;
-            if constexpr (Sm::kRaw) q = sm.raw[tr][cc];
-            else q = ld_state<LDCG>(&fin[o]);
+            const Vec4<S> q = ld_state<LDCG>(&fin[o]);
             const Vec4<R> p = sm.val[tr + 2][cc + 2];
             const Vec4<R> Fw = sm.fx[tr][cc], Fe = sm.fx[tr][cc + 1];
             const Vec4<R> Fs = sm.fy[tr][cc], Fn = sm.fy[tr + 1][cc];
@@ -570,15 +519,10 @@ __device__ __forceinline__ void tile_step(TileSmem<P, TX, TY, NT>& sm, const Cav
             const R dr = p.x, u = p.y, v = p.z, T = Tz + p.w;
             const R rho = one + dr;
             // Dt/dV sum_k F_k dS_k for mass, momentum, energy
-            R div0, div1, div2, div3;
-            if constexpr (sizeof(R) == 4) {
-                flux_div_f32(Fw, Fe, Fs, Fn, ax, ay, div0, div1, div2, div3);
-            } else {
-                div0 = ax * (Fe.x - Fw.x) + ay * (Fn.x - Fs.x);
-                div1 = ax * (Fe.y - Fw.y) + ay * (Fn.y - Fs.y);
-                div2 = ax * (Fe.z - Fw.z) + ay * (Fn.z - Fs.z);
-                div3 = ax * (Fe.w - Fw.w) + ay * (Fn.w - Fs.w);
-            }
+            const R div0 = ax * (Fe.x - Fw.x) + ay * (Fn.x - Fs.x);
+            const R div1 = ax * (Fe.y - Fw.y) + ay * (Fn.y - Fs.y);
+            const R div2 = ax * (Fe.z - Fw.z) + ay * (Fn.z - Fs.z);
+            const R div3 = ax * (Fe.w - Fw.w) + ay * (Fn.w - Fs.w);
             // Boussinesq source (Eq. 64, hot fluid rises) and body force
             const R src_x = rho * fxb;
             const R src_y = rho * (bg * (T - Tr) + fyb);
@@ -620,12 +564,11 @@ __device__ __forceinline__ void tile_step(TileSmem<P, TX, TY, NT>& sm, const Cav
 // the residual sums: a chain of about 32 + 165 + 55 instructions, where the
 // 32 x 4 tile's warps pass through some 750.  64^2: 29.4 -> 17.6 us per step.
 template <class P, int TX, int TY, int NT, bool LDCG>
-__device__ __forceinline__ void tile_step_flat(TileSmem<P, TX, TY, NT>& sm, const CavityDesc* dp,
-                                               int i0, int j0,
+__device__ __forceinline__ void tile_step_flat(TileSmem<P, TX, TY, NT>& sm, int i0, int j0,
                                                const Vec4<typename P::S>* __restrict__ fin,
-                                               Vec4<typename P::S>* __restrict__ fout,
-                                               bool lines_staged)
+                                               Vec4<typename P::S>* __restrict__ fout)
 {
+    const CavityDesc* const dp = &sm.desc;
     using Sm = TileSmem<P, TX, TY, NT>;
     using S = typename P::S;
     using R = typename P::R;
@@ -640,8 +583,7 @@ __device__ __forceinline__ void tile_step_flat(TileSmem<P, TX, TY, NT>& sm, cons
     const R Tz = P::val(qTz, 3);
     const bool interior = i0 >= 2 && j0 >= 2 && i0 + TX + 2 <= nx && j0 + TY + 2 <= ny;
 
-    // 1. mesh lines (unless staged) and the haloed tile
-    if (!lines_staged) stage_lines(sm, dp, i0, j0);
+    // 1. the haloed tile
     if (tid < BX * BY) {
         static_assert(BX * BY <= NT, "one box cell a thread");
         const int br = tid / BX, bc = tid - br * BX;
@@ -776,31 +718,62 @@ __device__ __forceinline__ void tile_step_flat(TileSmem<P, TX, TY, NT>& sm, cons
     if (lane == 0) sm.red[0][w] = w == 0 && bad ? R(NAN) : s;
 }
 
-// Threads of a tile block: two cells per thread in the update; one cell per
-// thread for the small FP64 tiles, whose point is to spread the narrow FP64
-// units' work over as many SM sub-partitions as possible; four threads per
-// cell for the flat one.
-template <class P, int TX, int TY>
-struct TileThreads {
-    static constexpr int value = TX * TY / 2;
+}  // namespace rtlbfs
+
+#include "rtlbfs_tile_pair.cuh"
+
+namespace rtlbfs {
+
+// Resident blocks per SM to compile for: FP32 as many as the tile buffers
+// allow with some 96 registers a thread (wide blocks: two, then one); FP64
+// takes the registers it needs, but no more than let two of its large blocks
+// share an SM (512^2 in 8-row tiles: 279 us per step at 130 registers, 254 at
+// 128).
+template <class P, int TX, int TY, int NT>
+struct MinBlocks {
+    static constexpr int value = NT == 256 ? 2 : 1;
 };
-template <int TX, int TY>
-struct TileThreads<StoreD, TX, TY> {
+template <int TX, int TY, int NT>
+struct MinBlocks<StoreQ, TX, TY, NT> {
+    static constexpr int smem = 227 * 1024 / ((int)sizeof(TileSmem<StoreQ, TX, TY, NT>) + 1024);
+    static constexpr int regs = 65536 / (NT * 96);
+    static constexpr int least = smem < regs ? smem : regs;
+    static constexpr int value = NT == 32 * (TY + 2)       ? 1
+                                 : NT == 32 * (TY / 2 + 1) ? 2
+                                 : least < 1               ? 1
+                                                           : least;
+};
+
+// Threads of a tile block.  FP32: as many warps as take one packed x-face
+// and one packed y-face each (WIDE = 1), twice (2) or half (0) as many.  FP64: two cells per
+// thread in the update; one cell per thread for the small tiles, whose point
+// is to spread the narrow FP64 units' work over as many SM sub-partitions as
+// possible; four threads per cell for the flat one.
+template <class P, int TX, int TY, int WIDE>
+struct TileThreads {
+    static constexpr int value =
+        32 * (WIDE == 2 ? TY + 2 : WIDE == 1 ? TY / 2 + 1 : TY / 2 < 1 ? 1 : (TY / 2 + 1) / 2);
+};
+template <int TX, int TY, int WIDE>
+struct TileThreads<StoreD, TX, TY, WIDE> {
     static constexpr int value = FlatTile<StoreD, TX, TY>::value ? 4 * TX * TY
                                  : TY <= 8                       ? TX * TY
                                                                  : TX * TY / 2;
 };
 
-// The step of one tile by the body its shape takes.
+// The step of one tile by the body its shape takes (after stage_tile and a
+// barrier).
 template <class P, int TX, int TY, int NT, int SCHEME, bool LDCG>
-__device__ __forceinline__ void run_tile(TileSmem<P, TX, TY, NT>& sm, const CavityDesc* dp, int i0,
-                                         int j0, const Vec4<typename P::S>* __restrict__ fin,
-                                         Vec4<typename P::S>* __restrict__ fout, bool lines_staged)
+__device__ __forceinline__ void run_tile(TileSmem<P, TX, TY, NT>& sm, int i0, int j0,
+                                         const Vec4<typename P::S>* __restrict__ fin,
+                                         Vec4<typename P::S>* __restrict__ fout)
 {
     if constexpr (FlatTile<P, TX, TY>::value)
-        tile_step_flat<P, TX, TY, NT, LDCG>(sm, dp, i0, j0, fin, fout, lines_staged);
+        tile_step_flat<P, TX, TY, NT, LDCG>(sm, i0, j0, fin, fout);
+    else if constexpr (sizeof(typename P::R) == 4)
+        tile_step_pair<TX, TY, NT, SCHEME, LDCG>(sm, i0, j0, fin, fout);
     else
-        tile_step<P, TX, TY, NT, SCHEME, LDCG>(sm, dp, i0, j0, fin, fout, lines_staged);
+        tile_step<P, TX, TY, NT, SCHEME, LDCG>(sm, i0, j0, fin, fout);
 }
 
 }  // namespace rtlbfs
