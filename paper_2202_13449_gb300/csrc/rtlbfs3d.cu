@@ -3,7 +3,8 @@
 // Nusselt reductions and the rtlbfs3d_* C ABI.
 //
 // Step kernel.  Work unit: a TX x TY tile of columns of one mesh and a chunk
-// of z-planes [k0, k1); one thread per column.  The block marches up the
+// of z-planes [k0, k1); one thread per column in FP64 (below), per pair of
+// columns in FP32 (rtlbfs3d_pair.cuh).  The block marches up the
 // chunk with a rolling window in shared memory -- the values of planes k,
 // k+1, k+2 on the tile plus a 2-cell ring, the Green-Gauss gradients of
 // planes k and k+1 on a 1-cell ring -- and per plane:
@@ -16,9 +17,9 @@
 //     predictor (Eqs. 46-48), corrector fluxes (Eqs. 57-59),
 //   the update of plane k with the Boussinesq source (Eq. 64) and the
 //     residual sums; the z-face below the next plane is the one just made.
-// The last unit to finish a step turns the sums into (R_u, R_T), advances
-// the step counter, flips the state buffer and decides whether the run is
-// done, so launches need no host round trip.  HBM sees one read and one
+// The head of the next launch turns the sums into (R_u, R_T), advances the
+// step counter, flips the state buffer and decides whether the run is done,
+// so launches need no host round trip.  HBM sees one read and one
 // write of the five fields per cell (halo re-reads hit L2).
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
@@ -36,6 +37,7 @@
 #include "rtlbfs3d_dev.cuh"
 #include "rtlbfs_dev.cuh"
 #include "rtlbfs_kernels.h"
+#include "rtlbfs_pair.cuh"
 
 namespace rtlbfs {
 extern std::atomic<long long> g_launches;
@@ -246,10 +248,6 @@ __device__ __forceinline__ void face3_frame(const Desc3& d, CellNT3<R>& L, R tau
     const R uw2 = wside >= 0 ? Cst<P>::uw(d, wside, a2) : R(0);
     if constexpr (SCH == 1) {
         face_flux3_tlbfs<R>(L, Rc, Tz + tauL, fl, keep, uw1, uw2, F);
-    } else if constexpr (sizeof(R) == 4) {  // FP32: the column stage in packed pairs
-        Cols3<R> c;
-        face3_columns_f32(L, Rc, fl, c);
-        face_flux3_columns<R>(c, Tz + tauL, fl, keep, uw1, uw2, F);
     } else {
         face_flux3<R>(L, Rc, Tz + tauL, fl, keep, uw1, uw2, F);
     }
@@ -471,69 +469,33 @@ __global__ void __launch_bounds__(TX* TY) step3_kernel(const Desc3* __restrict__
         // x- and y-faces of plane k
         const int vs = mod3(k), gs = mod2(k);
         constexpr int NXF = TY * (TX + 1), NYF = (TY + 1) * TX;
-        if constexpr (sizeof(R) == 4) {
-            // FP32: one loop (face t < NXF an x-face, else a y-face), so the
-            // face arithmetic is one copy of code and a thread's rounds cover
-            // both kinds; the fluxes come back in the face frame and are
-            // stored to their global components.  (FP64 keeps two loops: the
-            // shared copy would raise its registers past three blocks per SM.)
-            for (int t = tid; t < NXF + NYF; t += NT) {
-                const bool isx = t < NXF;
-                const int u = isx ? t : t - NXF;
-                const int fj = isx ? u / (TX + 1) : u / TX, fi = isx ? u % (TX + 1) : u % TX;
-                const int g = isx ? i0 + fi : j0 + fj;  // the face's index along its normal
-                if (isx ? (g > nx || j0 + fj >= ny) : (g > ny || i0 + fi >= nx)) continue;
-                const int ax = isx ? 0 : 1;
-                CellNT3<R> L, Rr;
-                R tl, tr;
-                take3<R>(sm, vs, gs, isx ? fj + 2 : fj + 1, isx ? fi + 1 : fi + 2, ax, L, tl);
-                take3<R>(sm, vs, gs, fj + 2, fi + 2, ax, Rr, tr);
-                const bool per = isx ? xper : yper;
-                const int n_ax = isx ? nx : ny;
-                const int ws = per ? -1 : (g == 0 ? 2 * ax : (g == n_ax ? 2 * ax + 1 : -1));
-                R F[5];
-                face3_frame<P, R, SCH>(d, L, tl, Rr, tr,
-                                       isx ? get_line(sm.xl, fi) : get_line(sm.yl, fj), Tz, ax,
-                                       ws, F);
-                // frame (rho, n, t1, t2, T) to global (rho, x, y, z, T): x-face
-                // n = x, t1 = y, t2 = z; y-face n = y, t1 = z, t2 = x
-                R* dst = isx ? &sm.fx[0][fj][fi] : &sm.fy[0][fj][fi];
-                const int qs = isx ? NXF : NYF;  // stride between components
-                dst[0] = F[0];
-                dst[(isx ? 1 : 2) * qs] = F[1];
-                dst[(isx ? 2 : 3) * qs] = F[2];
-                dst[(isx ? 3 : 1) * qs] = F[3];
-                dst[4 * qs] = F[4];
-            }
-        } else {
-            for (int t = tid; t < NXF; t += NT) {
-                const int fj = t / (TX + 1), fi = t % (TX + 1);
-                const int gx = i0 + fi;
-                if (gx > nx || j0 + fj >= ny) continue;
-                CellNT3<R> L, Rr;
-                R tl, tr;
-                take3<R>(sm, vs, gs, fj + 2, fi + 1, 0, L, tl);
-                take3<R>(sm, vs, gs, fj + 2, fi + 2, 0, Rr, tr);
-                const int ws = xper ? -1 : (gx == 0 ? 0 : (gx == nx ? 1 : -1));
-                R F[5];
-                face3<P, R, SCH>(d, L, tl, Rr, tr, get_line(sm.xl, fi), Tz, 0, ws, F);
+        for (int t = tid; t < NXF; t += NT) {
+            const int fj = t / (TX + 1), fi = t % (TX + 1);
+            const int gx = i0 + fi;
+            if (gx > nx || j0 + fj >= ny) continue;
+            CellNT3<R> L, Rr;
+            R tl, tr;
+            take3<R>(sm, vs, gs, fj + 2, fi + 1, 0, L, tl);
+            take3<R>(sm, vs, gs, fj + 2, fi + 2, 0, Rr, tr);
+            const int ws = xper ? -1 : (gx == 0 ? 0 : (gx == nx ? 1 : -1));
+            R F[5];
+            face3<P, R, SCH>(d, L, tl, Rr, tr, get_line(sm.xl, fi), Tz, 0, ws, F);
 #pragma unroll
-                for (int q = 0; q < 5; ++q) sm.fx[q][fj][fi] = F[q];
-            }
-            for (int t = tid; t < NYF; t += NT) {
-                const int fj = t / TX, fi = t % TX;
-                const int gy = j0 + fj;
-                if (gy > ny || i0 + fi >= nx) continue;
-                CellNT3<R> L, Rr;
-                R tl, tr;
-                take3<R>(sm, vs, gs, fj + 1, fi + 2, 1, L, tl);
-                take3<R>(sm, vs, gs, fj + 2, fi + 2, 1, Rr, tr);
-                const int ws = yper ? -1 : (gy == 0 ? 2 : (gy == ny ? 3 : -1));
-                R F[5];
-                face3<P, R, SCH>(d, L, tl, Rr, tr, get_line(sm.yl, fj), Tz, 1, ws, F);
+            for (int q = 0; q < 5; ++q) sm.fx[q][fj][fi] = F[q];
+        }
+        for (int t = tid; t < NYF; t += NT) {
+            const int fj = t / TX, fi = t % TX;
+            const int gy = j0 + fj;
+            if (gy > ny || i0 + fi >= nx) continue;
+            CellNT3<R> L, Rr;
+            R tl, tr;
+            take3<R>(sm, vs, gs, fj + 1, fi + 2, 1, L, tl);
+            take3<R>(sm, vs, gs, fj + 2, fi + 2, 1, Rr, tr);
+            const int ws = yper ? -1 : (gy == 0 ? 2 : (gy == ny ? 3 : -1));
+            R F[5];
+            face3<P, R, SCH>(d, L, tl, Rr, tr, get_line(sm.yl, fj), Tz, 1, ws, F);
 #pragma unroll
-                for (int q = 0; q < 5; ++q) sm.fy[q][fj][fi] = F[q];
-            }
+            for (int q = 0; q < 5; ++q) sm.fy[q][fj][fi] = F[q];
         }
         R Fu[5] = {R(0), R(0), R(0), R(0), R(0)};
         R c0[5];
@@ -598,6 +560,12 @@ __global__ void __launch_bounds__(TX* TY) step3_kernel(const Desc3* __restrict__
     __syncthreads();
     rtlbfs::add_sums(sm.red, NT / 32, run->acc[slot3]);  // the next launch tests them
 }
+
+}  // namespace rtlbfs3
+
+#include "rtlbfs3d_pair.cuh"
+
+namespace rtlbfs3 {
 
 // ---------------------------------------------------------------------------
 // FP64 Nusselt sums: one thread per face of a wall (or of the x mid-plane),
@@ -776,14 +744,49 @@ void build_lines(const std::vector<double>& f, bool periodic, double kappa, doub
     }
 }
 
-template <class P, int TX, int TY>
-cudaError_t launch_step(int units, int scheme, cudaStream_t s, const Desc3* d, CavityRun* c,
-                        int par)
+// The step kernel of a precision, tile and face stage: packed pairs in FP32.
+template <class P, int TX, int TY, int SCH>
+struct Step3 {
+    static constexpr auto fn = step3_kernel<P, TX, TY, SCH>;
+    static constexpr int threads = TX * TY;
+    static constexpr size_t smem = sizeof(Smem3<P, TX, TY>);
+};
+template <int TX, int TY, int SCH>
+struct Step3<StoreQ, TX, TY, SCH> {
+    static constexpr auto fn = step3_pair_kernel<TX, TY, SCH>;
+    static constexpr int threads = Smem3P<TX, TY>::NT;
+    static constexpr size_t smem = sizeof(Smem3P<TX, TY>);
+};
+
+// Blocks per SM are held at what one even round of the units needs, by asking
+// for the least shared memory that b + 1 blocks do not find: the blocks of the next step, launched while this one
+// drains, otherwise crowd onto the SMs that empty first. 64^3
+// in 32 x 8 tiles (256 units on 152 SMs): 32 us, 40 without.
+template <class K>
+cudaError_t launch_kernel3(int units, int sms, cudaStream_t s, const Desc3* d, CavityRun* c,
+                           int par)
 {
-    const size_t sm = sizeof(Smem3<P, TX, TY>);
-    if (scheme == 1)
-        return launch_chained(step3_kernel<P, TX, TY, 1>, units, TX * TY, sm, s, d, c, par);
-    return launch_chained(step3_kernel<P, TX, TY, 0>, units, TX * TY, sm, s, d, c, par);
+    const size_t b = (size_t)(units + sms - 1) / sms;
+    const size_t smem = std::max(K::smem, (228 * 1024 / (b + 1) - 1024) / 128 * 128 + 128);
+    return launch_chained(K::fn, units, K::threads, smem, s, d, c, par);
+}
+
+template <class P, int TX, int TY>
+cudaError_t launch_step(int units, int scheme, int sms, cudaStream_t s, const Desc3* d,
+                        CavityRun* c, int par)
+{
+    if (scheme == 1) return launch_kernel3<Step3<P, TX, TY, 1>>(units, sms, s, d, c, par);
+    return launch_kernel3<Step3<P, TX, TY, 0>>(units, sms, s, d, c, par);
+}
+
+template <class K>
+cudaError_t prepare_kernel3(int* occ)
+{
+    cudaError_t e =
+        cudaFuncSetAttribute(K::fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, K::fn, K::threads, K::smem);
+    return e;
 }
 
 // shared-memory opt-in and resident blocks per SM of both face stages
@@ -791,19 +794,8 @@ cudaError_t launch_step(int units, int scheme, cudaStream_t s, const Desc3* d, C
 template <class P, int TX, int TY>
 cudaError_t prepare_kernel(int occ[2])
 {
-    const size_t sm = sizeof(Smem3<P, TX, TY>);
-    cudaError_t e = cudaFuncSetAttribute(step3_kernel<P, TX, TY, 0>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(step3_kernel<P, TX, TY, 1>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[0], step3_kernel<P, TX, TY, 0>,
-                                                          TX * TY, sm);
-    if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[1], step3_kernel<P, TX, TY, 1>,
-                                                          TX * TY, sm);
-    return e;
+    cudaError_t e = prepare_kernel3<Step3<P, TX, TY, 0>>(&occ[0]);
+    return e == cudaSuccess ? prepare_kernel3<Step3<P, TX, TY, 1>>(&occ[1]) : e;
 }
 
 }  // namespace rtlbfs3
@@ -903,16 +895,32 @@ void decompose(rtlbfs3d_ctx* h, Desc3& d)
     d.tiles_y = (h->n[1] + TY - 1) / TY;
     int kc = h->kchunk_req;
     if (kc <= 0) {
-        const long long slots =
-            (long long)std::max(1, h->sms) * std::max(1, h->occ[h->tile][h->scheme]);
+        // The chunk of the least modelled time.  A unit takes its planes and
+        // the like of `extra` more for the planes below it; units on an SM at
+        // once slow each other by `slow` per unit beyond the first: in FP32
+        // by 8 % a warp (latency hides in the others' gaps), in FP64 by the
+        // share of the FP64 units each needs.  80^3 in 16 x 8 tiles, time
+        // over that of the pick, modelled and measured: FP32 (pick 7 planes,
+        // 48 us) 4 planes 1.22 and 1.26, 8 planes 1.11 and 1.11; FP64 (pick
+        // 9, 1336 us) 4 planes 1.15 and 1.16, 8 planes 1.27 and 1.14.  Where
+        // the mesh leaves SMs idle the pick is a plane or two: 16^3 12 us
+        // (FP64 92), against 22 (269) with chunks of 4.
+        const bool fp64 = h->precision == RTLBFS_FP64;
+        const int occ = std::max(1, h->occ[h->tile][h->scheme]), sms = std::max(1, h->sms);
         const long long per_plane = (long long)d.tiles_x * d.tiles_y;
-        long long chunks = std::max(1LL, (slots + per_plane - 1) / per_plane);
-        kc = (int)std::max(4LL, (h->n[2] + chunks - 1) / chunks);
-        // small meshes (a wave holds two planes of columns or more): the
-        // shortest chunk of at least 4 planes whose units fit one wave, so
-        // that no short second wave follows
-        if (2 * per_plane <= slots)
-            while (kc < h->n[2] && per_plane * ((h->n[2] + kc - 1) / kc) > slots) ++kc;
+        const double warps = TX * TY / (fp64 ? 32 : 64), extra = fp64 ? 0.55 : 1.5;
+        const double slow = fp64 ? 0.35 + 0.0875 * warps : 0.08 * warps;
+        auto busy = [&](long long m) { return m > 0 ? 1.0 + slow * (m - 1) : 0.0; };
+        double best = INFINITY;
+        for (int k = 1; k <= h->n[2]; ++k) {
+            const long long units = per_plane * ((h->n[2] + k - 1) / k);
+            const long long b = (units + sms - 1) / sms;  // units of the busiest SM
+            const double t = (k + extra) * ((b / occ) * busy(occ) + busy(b % occ));
+            if (t < best) {
+                best = t;
+                kc = k;
+            }
+        }
     }
     kc = std::min(kc, h->n[2]);
     d.kchunk = kc;
@@ -1006,18 +1014,18 @@ cudaError_t launch_one(rtlbfs3d_ctx* h, cudaStream_t s, int par)
 {
     const int units = h->desc.units;
     rtlbfs::g_launches++;
-    const int sc = h->scheme;
+    const int sc = h->scheme, sms = std::max(1, h->sms);
     if (h->precision == RTLBFS_FP64) {
         switch (h->tile) {
-        case 0: return launch_step<StoreD, 32, 4>(units, sc, s, h->d_desc, h->d_ctl, par);
-        case 1: return launch_step<StoreD, 16, 8>(units, sc, s, h->d_desc, h->d_ctl, par);
-        default: return launch_step<StoreD, 32, 8>(units, sc, s, h->d_desc, h->d_ctl, par);
+        case 0: return launch_step<StoreD, 32, 4>(units, sc, sms, s, h->d_desc, h->d_ctl, par);
+        case 1: return launch_step<StoreD, 16, 8>(units, sc, sms, s, h->d_desc, h->d_ctl, par);
+        default: return launch_step<StoreD, 32, 8>(units, sc, sms, s, h->d_desc, h->d_ctl, par);
         }
     }
     switch (h->tile) {
-    case 0: return launch_step<StoreQ, 32, 4>(units, sc, s, h->d_desc, h->d_ctl, par);
-    case 1: return launch_step<StoreQ, 16, 8>(units, sc, s, h->d_desc, h->d_ctl, par);
-    default: return launch_step<StoreQ, 32, 8>(units, sc, s, h->d_desc, h->d_ctl, par);
+    case 0: return launch_step<StoreQ, 32, 4>(units, sc, sms, s, h->d_desc, h->d_ctl, par);
+    case 1: return launch_step<StoreQ, 16, 8>(units, sc, sms, s, h->d_desc, h->d_ctl, par);
+    default: return launch_step<StoreQ, 32, 8>(units, sc, sms, s, h->d_desc, h->d_ctl, par);
     }
 }
 

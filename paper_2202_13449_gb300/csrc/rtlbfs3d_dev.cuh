@@ -57,11 +57,10 @@ struct CellNT3 {
 //   d_t f   = 2 (odd part in t at a = 0),  dd_t f = 2 (t^2 coefficient),
 //   dd_t1t2 f = 4 (b c coefficient),
 //   dd_nt f = 2 (odd part in t on a = +1, minus that on a = -1):
-// the same numbers with a third fewer operations (280 a face against 435
+// the same numbers with a third fewer operations (281 a face against 435
 // for products at the 19 nodes), and without the cancellation of the node
 // differences.  FP64 runs at the FMA rate, so there the step follows the
-// count: 20 steps of an 80^3 mesh and the download, FP64, 34.8 -> 29.5 ms;
-// FP32, bound by its shared-memory phases, is unchanged (21.8 ms for 300).
+// count: 20 steps of an 80^3 mesh and the download, FP64, 34.8 -> 29.0 ms.
 //
 // The first stage, face3_columns, forms the coefficients C, S1, S2 of the
 // five primitives on the three columns (A: a = -1, M: a = 0, B: a = +1);
@@ -127,10 +126,10 @@ __host__ __device__ __forceinline__ SideCol3<V> side_column3(const V C[5], const
     return s;
 }
 
-template <typename V>
-__host__ __device__ __forceinline__ void face_flux3_columns(const Cols3<V>& c, V Tbar,
-                                                           const FaceLine<V>& fl, V keep, V uw1,
-                                                           V uw2, V F[5])
+// wall(mn, m1, m2, rho): the wall rule on the predicted momenta.
+template <typename V, class W>
+__host__ __device__ __forceinline__ void face_flux3_wall(const Cols3<V>& c, V Tbar,
+                                                        const FaceLine<V>& fl, W wall, V F[5])
 {
     using T = vtraits<V>;
     const V zero = T::bc(0.0), half = T::bc(0.5), one = T::bc(1.0);
@@ -219,10 +218,7 @@ __host__ __device__ __forceinline__ void face_flux3_columns(const Cols3<V>& c, V
     es = vfma(hcs2, vfma(two, eq[0] + eq[1], vfma(m2, e0, se)), es);
 
     const V rho_s = one + drs;
-    // wall faces: no mass through the wall, the wall's tangential velocity
-    ms[0] = ms[0] * keep;
-    ms[1] = vfma(keep, ms[1], rho_s * uw1);
-    ms[2] = vfma(keep, ms[2], rho_s * uw2);
+    wall(ms[0], ms[1], ms[2], rho_s);
     const V inv = T::rcp(rho_s);
     const V un_s = ms[0] * inv;
     const V taus = (es - drs * Tbar) * inv;  // T* - Tbar
@@ -254,44 +250,14 @@ __host__ __device__ __forceinline__ void face_flux3(const CellNT3<V>& L, const C
 {
     Cols3<V> c;
     face3_columns<V>(L, Rc, fl, c);
-    face_flux3_columns<V>(c, Tbar, fl, keep, uw1, uw2, F);
-}
-
-// face3_columns in FP32, components (0, 1) and (2, 3) in packed FP32x2 pairs
-// (component 4 alone): the same operations, bit for bit.
-__device__ __forceinline__ void face3_columns_f32(const CellNT3<float>& L, const CellNT3<float>& Rc,
-                                                  const FaceLine<float>& fl, Cols3<float>& c)
-{
-    const float h = fl.h;
-    const float wL = fl.cL + h, mwR = fl.cR - h, hh = h * 0.5f;
-    const float2 cL2 = make_float2(fl.cL, fl.cL), cR2 = make_float2(fl.cR, fl.cR);
-    const float2 wL2 = make_float2(wL, wL), mwR2 = make_float2(mwR, mwR);
-    const float2 h2 = make_float2(h, h), hh2 = make_float2(hh, hh);
-    const float2 half2 = make_float2(0.5f, 0.5f);
-    auto pr = [](const float* a, int i) { return make_float2(a[2 * i], a[2 * i + 1]); };
-    auto put = [](float* d, int i, float2 v) {
-        d[2 * i] = v.x;
-        d[2 * i + 1] = v.y;
-    };
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        const float2 q = pr(L.q, i), gn = pr(L.gn, i), g1 = pr(L.g1, i), g2 = pr(L.g2, i);
-        const float2 qr = pr(Rc.q, i), gnr = pr(Rc.gn, i), g1r = pr(Rc.g1, i), g2r = pr(Rc.g2, i);
-        put(c.A, i, __ffma2_rn(gn, cL2, q));
-        put(c.A1, i, __fmul2_rn(g1, h2));
-        put(c.A2, i, __fmul2_rn(g2, h2));
-        put(c.B, i, __ffma2_rn(gnr, cR2, qr));
-        put(c.B1, i, __fmul2_rn(g1r, h2));
-        put(c.B2, i, __fmul2_rn(g2r, h2));
-        put(c.M, i, __fmul2_rn(half2, __fadd2_rn(__ffma2_rn(gn, wL2, q), __ffma2_rn(gnr, mwR2, qr))));
-        put(c.M1, i, __fmul2_rn(hh2, __fadd2_rn(g1, g1r)));
-        put(c.M2, i, __fmul2_rn(hh2, __fadd2_rn(g2, g2r)));
-    }
-    c.A[4] = fmaf(L.gn[4], fl.cL, L.q[4]);
-    c.B[4] = fmaf(Rc.gn[4], fl.cR, Rc.q[4]);
-    c.M[4] = 0.5f * (fmaf(L.gn[4], wL, L.q[4]) + fmaf(Rc.gn[4], mwR, Rc.q[4]));
-    c.M1[4] = hh * (L.g1[4] + Rc.g1[4]);
-    c.M2[4] = hh * (L.g2[4] + Rc.g2[4]);
+    // wall faces: no mass through the wall, the wall's tangential velocity
+    face_flux3_wall<V>(c, Tbar, fl,
+                       [&](V& mn, V& m1, V& m2, V rho) {
+                           mn = mn * keep;
+                           m1 = vfma(keep, m1, rho * uw1);
+                           m2 = vfma(keep, m2, rho * uw2);
+                       },
+                       F);
 }
 
 // The original TLBFS face stage (Section 2.2) with D3Q19, from the same
@@ -303,22 +269,21 @@ __device__ __forceinline__ void face3_columns_f32(const CellNT3<float>& L, const
 // Equilibria are carried as deviations f_i - w_i and g_i - w_i Tbar; the
 // constants cancel in every moment used except the pressure c_s^2 of the
 // normal momentum flux, which is dropped as in face_flux3.
-template <typename V>
-__host__ __device__ __forceinline__ void face_flux3_tlbfs(const CellNT3<V>& L, const CellNT3<V>& Rc,
-                                                         V Tbar, const FaceLine<V>& fl, V keep,
-                                                         V uw1, V uw2, V F[5])
+//
+// The moments of the predicted state's equilibria that a flux needs are
+// exact (c_s^2 rho + rho u_n u_n, rho u_n u_t, rho u_n T), so only the
+// nodes' equilibria are formed one by one, without their weights, and summed
+// by weight and sign (as in the 2D stage).
+template <typename V, class W>
+__host__ __device__ __forceinline__ void face_flux3_tlbfs_wall(const CellNT3<V>& L,
+                                                              const CellNT3<V>& Rc, V Tbar,
+                                                              const FaceLine<V>& fl, W wall, V F[5])
 {
     using T = vtraits<V>;
-    const V zero = T::bc(0.0), half = T::bc(0.5), one = T::bc(1.0), three = T::bc(3.0);
-    const V c45 = T::bc(4.5), mc15 = T::bc(-1.5), six = T::bc(6.0);
-    // D3Q19 (Eq. 5) in the face frame: the set is the same in every frame
-    constexpr int en[19] = {0, 1, -1, 0, 0, 0, 0, 1, -1, 1, -1, 1, -1, 1, -1, 0, 0, 0, 0};
-    constexpr int e1[19] = {0, 0, 0, 1, -1, 0, 0, 1, 1, -1, -1, 0, 0, 0, 0, 1, -1, 1, -1};
-    constexpr int e2[19] = {0, 0, 0, 0, 0, 1, -1, 0, 0, 0, 0, 1, 1, -1, -1, 1, 1, -1, -1};
+    const V one = T::bc(1.0), c45 = T::bc(4.5), mc15 = T::bc(-1.5), cs2 = T::bc(1.0 / 3.0);
     const V w0 = T::bc(1.0 / 3.0), w1 = T::bc(1.0 / 18.0), w2 = T::bc(1.0 / 36.0);
-    const V h = fl.h;
+    const V half = T::bc(0.5), h = fl.h;
     const V wL = fl.cL + h, mwR = fl.cR - h;
-    const V hh = h * half;
     // columns a = -1 (left plane), 0 (mean), +1 (right plane): value + slopes in t1, t2
     V C[3][5], S1[3][5], S2[3][5];
 #pragma unroll
@@ -330,83 +295,114 @@ __host__ __device__ __forceinline__ void face_flux3_tlbfs(const CellNT3<V>& L, c
         S1[2][k] = Rc.g1[k] * h;
         S2[2][k] = Rc.g2[k] * h;
         C[1][k] = half * (vfma(L.gn[k], wL, L.q[k]) + vfma(Rc.gn[k], mwR, Rc.q[k]));
-        S1[1][k] = hh * (L.g1[k] + Rc.g1[k]);
-        S2[1][k] = hh * (L.g2[k] + Rc.g2[k]);
+        S1[1][k] = half * (S1[0][k] + S1[2][k]);
+        S2[1][k] = half * (S2[0][k] + S2[2][k]);
     }
-    // (a), (b): equilibria at the nodes -e_i and their moments
-    V df[19], dg[19];
-    V drs = zero, mn = zero, m1 = zero, m2 = zero, es = zero;
-#pragma unroll
-    for (int i = 0; i < 19; ++i) {
-        const int a = 1 - en[i], b = -e1[i], c = -e2[i];  // column, offsets along t1, t2
+    // equilibria of direction (en, e1, e2) at the node opposite, over their
+    // weights: f_i / w_i - 1 = drho + rho (3 eu + 4.5 eu^2 - 1.5 u^2), and
+    // g_i / w_i - Tbar
+    auto equil = [&](int en, int e1, int e2, V& f, V& g) {
+        const int a = 1 - en;
         V q[5];
 #pragma unroll
         for (int k = 0; k < 5; ++k) {
             V x = C[a][k];
-            if (b > 0) x = x + S1[a][k];
-            if (b < 0) x = x - S1[a][k];
-            if (c > 0) x = x + S2[a][k];
-            if (c < 0) x = x - S2[a][k];
+            if (e1 < 0) x = x + S1[a][k];
+            if (e1 > 0) x = x - S1[a][k];
+            if (e2 < 0) x = x + S2[a][k];
+            if (e2 > 0) x = x - S2[a][k];
             q[k] = x;
         }
-        const V w = i == 0 ? w0 : (i < 7 ? w1 : w2);
-        V eu = zero;
-        if (en[i] > 0) eu = eu + q[1];
-        if (en[i] < 0) eu = eu - q[1];
-        if (e1[i] > 0) eu = eu + q[2];
-        if (e1[i] < 0) eu = eu - q[2];
-        if (e2[i] > 0) eu = eu + q[3];
-        if (e2[i] < 0) eu = eu - q[3];
-        const V usq = vfma(q[1], q[1], vfma(q[2], q[2], q[3] * q[3]));
-        const V rho = one + q[0];
-        // f_i - w_i = w_i (drho + rho (3 eu + 4.5 eu^2 - 1.5 u^2))
-        df[i] = w * vfma(rho, vfma(eu, vfma(c45, eu, three), mc15 * usq), q[0]);
-        // rho T - Tbar at the node, and g_i - w_i Tbar
-        const V e_node = vfma(q[0], Tbar + q[4], q[4]);
-        dg[i] = w * vfma(three * eu, Tbar + e_node, e_node);
-        drs = drs + df[i];
-        if (en[i] > 0) mn = mn + df[i];
-        if (en[i] < 0) mn = mn - df[i];
-        if (e1[i] > 0) m1 = m1 + df[i];
-        if (e1[i] < 0) m1 = m1 - df[i];
-        if (e2[i] > 0) m2 = m2 + df[i];
-        if (e2[i] < 0) m2 = m2 - df[i];
-        es = es + dg[i];
-    }
+        const V e = vfma(q[0], Tbar + q[4], q[4]);
+        const V u2 = mc15 * vfma(q[1], q[1], vfma(q[2], q[2], q[3] * q[3]));
+        if (en == 0 && e1 == 0 && e2 == 0) {
+            f = vfma(one + q[0], u2, q[0]);
+            g = e;
+            return;
+        }
+        // eu = sign * s, s one velocity or the sum or difference of two
+        const int sg = en != 0 ? en : (e1 != 0 ? e1 : e2);
+        V s = en != 0 ? q[1] : (e1 != 0 ? q[2] : q[3]);
+        if (en != 0 && e1 != 0) s = en == e1 ? s + q[2] : s - q[2];
+        if ((en != 0 || e1 != 0) && e2 != 0) s = sg == e2 ? s + q[3] : s - q[3];
+        const V three = T::bc(sg > 0 ? 3.0 : -3.0);
+        f = vfma(one + q[0], vfma(s, vfma(c45, s, three), u2), q[0]);
+        g = vfma(three * s, Tbar + e, e);
+    };
+    // opposite directions together: sum and difference of f and g
+    auto both = [&](int en, int e1, int e2, V& sf, V& df, V& sg, V& dg) {
+        V fp, gp, fm, gm;
+        equil(en, e1, e2, fp, gp);
+        equil(-en, -e1, -e2, fm, gm);
+        sf = fp + fm;
+        df = fp - fm;
+        sg = gp + gm;
+        dg = gp - gm;
+    };
+    // the predicted variables as moments, with those of the fluxes
+    V f0, g0, sf, df, sg, dg;
+    equil(0, 0, 0, f0, g0);
+    V An, Dn, Gn, En;  // axis directions, normal
+    both(1, 0, 0, An, Dn, Gn, En);
+    V S1s = An, G1s = Gn;
+    V D1, D2;
+    both(0, 1, 0, sf, D1, sg, dg);
+    S1s = S1s + sf;
+    G1s = G1s + sg;
+    both(0, 0, 1, sf, D2, sg, dg);
+    S1s = S1s + sf;
+    G1s = G1s + sg;
+    // edge directions: d1 = (n, t1), d2 = (n, t2), d3 = (t1, t2)
+    V sa, da, ga, ea, sb, db, gb, eb;
+    both(1, 1, 0, sa, da, ga, ea);
+    both(1, -1, 0, sb, db, gb, eb);
+    V Sn2 = sa + sb, G2s = ga + gb, mn2 = da + db, m12 = da - db, En2 = ea + eb;
+    const V Xn1e = sa - sb;
+    both(1, 0, 1, sa, da, ga, ea);
+    both(1, 0, -1, sb, db, gb, eb);
+    Sn2 = Sn2 + (sa + sb);
+    G2s = G2s + (ga + gb);
+    mn2 = mn2 + (da + db);
+    V m22 = da - db;
+    En2 = En2 + (ea + eb);
+    const V Xn2e = sa - sb;
+    both(0, 1, 1, sa, da, ga, ea);
+    both(0, 1, -1, sb, db, gb, eb);
+    const V S2s = Sn2 + (sa + sb);
+    G2s = G2s + (ga + gb);
+    m12 = m12 + (da + db);
+    m22 = m22 + (da - db);
+    const V drs = vfma(w0, f0, vfma(w1, S1s, w2 * S2s));
+    const V es = vfma(w0, g0, vfma(w1, G1s, w2 * G2s));
+    V mn = vfma(w1, Dn, w2 * mn2), m1 = vfma(w1, D1, w2 * m12), m2 = vfma(w1, D2, w2 * m22);
+    const V Xnn = vfma(w1, An, w2 * Sn2), Xn1 = w2 * Xn1e, Xn2 = w2 * Xn2e;
+    const V Qn = vfma(w1, En, w2 * En2);
     const V rho_s = one + drs;
-    mn = mn * keep;
-    const V wallr = (one - keep) * rho_s;
-    m1 = vfma(keep, m1, wallr * uw1);
-    m2 = vfma(keep, m2, wallr * uw2);
-    const V inv = T::rcp(rho_s);
-    const V un = mn * inv, u1 = m1 * inv, u2 = m2 * inv;
-    const V usq_s = vfma(un, un, vfma(u1, u1, u2 * u2));
-    // (c) fluxes along +n; 1/2 - tau = -3 nu / h = 6 (-nu / 2h) (Eqs. 9-10)
-    const V cf = six * fl.m_nu_2h, cg = six * fl.m_chi_2h;
-    V Fnn = zero, Fn1 = zero, Fn2 = zero, Q = zero;
-#pragma unroll
-    for (int i = 0; i < 19; ++i) {
-        if (en[i] == 0) continue;  // no flux along n
-        const V w = i < 7 ? w1 : w2;
-        V eu = en[i] > 0 ? un : zero - un;
-        if (e1[i] > 0) eu = eu + u1;
-        if (e1[i] < 0) eu = eu - u1;
-        if (e2[i] > 0) eu = eu + u2;
-        if (e2[i] < 0) eu = eu - u2;
-        const V dfs = w * vfma(rho_s, vfma(eu, vfma(c45, eu, three), mc15 * usq_s), drs);
-        const V dgs = w * vfma(three * eu, Tbar + es, es);
-        const V pf = vfma(cf, dfs - df[i], dfs);  // f* + (1/2 - tau_f)(f* - f_node)
-        const V pg = vfma(cg, dgs - dg[i], dgs);
-        Fnn = Fnn + pf;  // e_n^2 = 1
-        if (e1[i] != 0) Fn1 = (en[i] * e1[i] > 0) ? Fn1 + pf : Fn1 - pf;
-        if (e2[i] != 0) Fn2 = (en[i] * e2[i] > 0) ? Fn2 + pf : Fn2 - pf;
-        Q = en[i] > 0 ? Q + pg : Q - pg;
-    }
+    wall(mn, m1, m2, rho_s);
+    const V un = mn * T::rcp(rho_s);
+    // fluxes along +n: the moments of the predicted equilibria plus the
+    // non-equilibrium parts; 1/2 - tau = -3 nu / h = 6 (-nu / 2h) (Eqs. 9-10)
+    const V cf = T::bc(6.0) * fl.m_nu_2h, cg = T::bc(6.0) * fl.m_chi_2h;
+    const V Fnn = vfma(mn, un, cs2 * drs), Fn1 = m1 * un, Fn2 = m2 * un, Q = un * (Tbar + es);
     F[0] = mn;
-    F[1] = Fnn;
-    F[2] = Fn1;
-    F[3] = Fn2;
-    F[4] = Q;
+    F[1] = vfma(cf, Fnn - Xnn, Fnn);
+    F[2] = vfma(cf, Fn1 - Xn1, Fn1);
+    F[3] = vfma(cf, Fn2 - Xn2, Fn2);
+    F[4] = vfma(cg, Q - Qn, Q);
+}
+
+template <typename V>
+__host__ __device__ __forceinline__ void face_flux3_tlbfs(const CellNT3<V>& L, const CellNT3<V>& Rc,
+                                                         V Tbar, const FaceLine<V>& fl, V keep,
+                                                         V uw1, V uw2, V F[5])
+{
+    face_flux3_tlbfs_wall<V>(L, Rc, Tbar, fl,
+                             [&](V& mn, V& m1, V& m2, V rho) {
+                                 mn = mn * keep;
+                                 m1 = vfma(keep, m1, rho * uw1);
+                                 m2 = vfma(keep, m2, rho * uw2);
+                             },
+                             F);
 }
 
 }  // namespace rtlbfs3
