@@ -10,7 +10,8 @@
 // coefficients of Eqs. 9-10 (FaceRec); per cell, the four Green-Gauss
 // coefficients w_f S_f / A of Eqs. 55-56 (CellGrad).
 //
-// Step kernel.  Work unit: a TX x TY tile of cells.  Before it waits for the
+// Step kernel (FP64 below; FP32, in pairs of cells, in rtlbfs_curv_pair.cuh).
+// Work unit: a TX x TY tile of cells.  Before it waits for the
 // previous step's grid, a block starts asynchronous copies of the tile's
 // geometry into shared memory (it never changes between steps); then:
 //   1. the tile plus a 2-cell ring of (rho - 1, u, v, T - Tz), ghosts
@@ -23,8 +24,9 @@
 //      into the values, then the rectilinear face template face_flux (Eq. 29
 //      nodes, Eqs. 46-48, Eqs. 57-59) and the fluxes rotated back;
 //   4. the update with the face lengths and areas, the Boussinesq source
-//      along the gravity direction, and the residual sums; the last unit
-//      finalises the step (residual, step counter, buffer flip, stop test).
+//      along the gravity direction, and the residual sums; the head of the
+//      next launch finalises the step (residual, step counter, buffer flip,
+//      stop test).
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
 
@@ -40,6 +42,7 @@
 #include "rtlbfs_curv.h"
 #include "rtlbfs_dev.cuh"
 #include "rtlbfs_kernels.h"
+#include "rtlbfs_pair.cuh"
 
 namespace rtlbfs {
 extern std::atomic<long long> g_launches;
@@ -52,7 +55,6 @@ using rtlbfs::chain_sync;
 using rtlbfs::launch_chained;
 using rtlbfs::FaceLine;
 using rtlbfs::face_flux;
-using rtlbfs::face_flux_columns;
 using rtlbfs::kConverged;
 using rtlbfs::kDiverged;
 using rtlbfs::kMaxSteps;
@@ -127,6 +129,7 @@ __device__ __forceinline__ T ld_vec(const T* p)
 
 struct DescC {
     int ni, nj, per, tiles_x, tiles_y, units;
+    int pair_rows;  // FP32: rows of a strip as stored
     int kind[4];
     double gdir[2], force[2], beta_g, T_ref, dt;
     float f_gdir[2], f_force[2], f_beta_g, f_T_ref, f_dt;
@@ -135,6 +138,8 @@ struct DescC {
     double d_inf[4];  // free stream (rho - 1, u, v, T)
     float f_inf[4];
     void* rec[2];                          // Vec4<S>[cells]
+    // FP64: the types noted; FP32: strips of PairFaceI[pair_rows],
+    // PairFaceJ[pair_rows + 1], PairRow[pair_rows + 2], float[pair_rows][kPairX]
     const void* fri;                       // FaceRec<R>[nj][ni+1]
     const void* frj;                       // FaceRec<R>[nj+1][ni]
     const void* cg;                        // CellGrad<R>[cells]
@@ -243,39 +248,6 @@ __host__ __device__ __forceinline__ void mirror_grad_c(int kind, R nx, R ny, R g
     }
 }
 
-// face_columns in FP32 on face-frame cells whose components were formed
-// in registers (a curvilinear face's rotated values): pairs (rho, u_n) and
-// (u_t, T) in packed FP32x2 instructions.
-__device__ __forceinline__ void face_columns_nt_f32(const rtlbfs::CellNT<float>& L, const rtlbfs::CellNT<float>& Rc,
-                                                    const FaceLine<float>& fl, float A[4],
-                                                    float Na[4], float M[4], float D[4],
-                                                    float B[4], float Sb[4])
-{
-    const float h = fl.h;
-    const float wL = fl.cL + h, mwR = fl.cR - h;
-    const float2 cL2 = make_float2(fl.cL, fl.cL), cR2 = make_float2(fl.cR, fl.cR);
-    const float2 wL2 = make_float2(wL, wL), mwR2 = make_float2(mwR, mwR);
-    const float2 h2 = make_float2(h, h), mh2 = make_float2(-h, -h), half2 = make_float2(0.5f, 0.5f);
-    const float2 m1 = make_float2(-1.0f, -1.0f);
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        const int k = 2 * i;
-        const float2 ql = make_float2(L.q[k], L.q[k + 1]), qr = make_float2(Rc.q[k], Rc.q[k + 1]);
-        const float2 nl = make_float2(L.gn[k], L.gn[k + 1]), nr = make_float2(Rc.gn[k], Rc.gn[k + 1]);
-        const float2 tl = make_float2(L.gt[k], L.gt[k + 1]), tr = make_float2(Rc.gt[k], Rc.gt[k + 1]);
-        const float2 a = __ffma2_rn(nl, cL2, ql), na = __fmul2_rn(tl, mh2);
-        const float2 b = __ffma2_rn(nr, cR2, qr), sb = __fmul2_rn(tr, h2);
-        const float2 m = __fmul2_rn(half2, __fadd2_rn(__ffma2_rn(nl, wL2, ql), __ffma2_rn(nr, mwR2, qr)));
-        const float2 d = __ffma2_rn(na, m1, sb);
-        A[k] = a.x, A[k + 1] = a.y;
-        Na[k] = na.x, Na[k + 1] = na.y;
-        B[k] = b.x, B[k + 1] = b.y;
-        Sb[k] = sb.x, Sb[k + 1] = sb.y;
-        M[k] = m.x, M[k + 1] = m.y;
-        D[k] = d.x, D[k + 1] = d.y;
-    }
-}
-
 // One face: values v[4] = (rho - 1, u, v, T - Tz) and gradients g[8] of the
 // two cells, the face geometry, the wall flag and tangential wall velocity.
 // Returns the fluxes times the face length in x, y components.
@@ -320,18 +292,7 @@ __host__ __device__ __forceinline__ void face_c(const R vL[4], const R gL[8], co
     fl.pad = R(0);
     const R uwt = uwx * tx + uwy * ty;
     R F[4];
-#ifdef __CUDA_ARCH__
-    constexpr bool packed = sizeof(R) == 4;  // FP32 on the device: packed column stage
-#else
-    constexpr bool packed = false;
-#endif
-    if constexpr (packed) {
-        R A[4], Na[4], M[4], D[4], B[4], Sb[4];
-        face_columns_nt_f32(L, Rr, fl, A, Na, M, D, B, Sb);
-        face_flux_columns<R>(A, Na, M, D, B, Sb, Tz + tauL, fl, keep, uwt, F);
-    } else {
-        face_flux<R>(L, Rr, Tz + tauL, fl, keep, uwt, F);
-    }
+    face_flux<R>(L, Rr, Tz + tauL, fl, keep, uwt, F);
     out[0] = F[0] * fg.len;
     out[1] = (F[1] * nx + F[2] * tx) * fg.len;
     out[2] = (F[1] * ny + F[2] * ty) * fg.len;
@@ -343,11 +304,6 @@ __device__ __forceinline__ void cp_async16(void* sdst, const void* gsrc)
 {
     const unsigned a = (unsigned)__cvta_generic_to_shared(sdst);
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(a), "l"(gsrc) : "memory");
-}
-__device__ __forceinline__ void cp_async_n(void* sdst, const void* gsrc, float*)
-{
-    const unsigned a = (unsigned)__cvta_generic_to_shared(sdst);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(a), "l"(gsrc) : "memory");
 }
 __device__ __forceinline__ void cp_async_n(void* sdst, const void* gsrc, double*)
 {
@@ -593,6 +549,12 @@ __global__ void __launch_bounds__(TX* TY) curv_step_kernel(const DescC* __restri
     rtlbfs::add_sums(sm.red, NT / 32, run->acc[slot3]);  // the next launch tests them
 }
 
+}  // namespace rtlbfsc
+
+#include "rtlbfs_curv_pair.cuh"
+
+namespace rtlbfsc {
+
 // ---------------------------------------------------------------------------
 // FP64 heat through side 2 or 3, one thread per face.
 // ---------------------------------------------------------------------------
@@ -684,24 +646,38 @@ __global__ void curv_heat_kernel(const DescC* __restrict__ dp, int cur, int jfac
 constexpr int kTileX = 32;
 constexpr int kGraphSteps = 32;
 
+// The step kernel of a precision and tile height: packed pairs in FP32.
+template <class P, int TY>
+struct StepC {
+    static constexpr auto fn = curv_step_kernel<P, kTileX, TY>;
+    static constexpr int threads = kTileX * TY;
+    static constexpr size_t smem = sizeof(SmemC<P, kTileX, TY>);
+};
+template <int TY>
+struct StepC<StoreQ, TY> {
+    static_assert(kTileX == kPairX, "strips of the tile width");
+    static constexpr auto fn = curv_pair_kernel<TY>;
+    static constexpr int threads = SmemCP<TY>::NT;
+    static constexpr size_t smem = sizeof(SmemCP<TY>);
+};
+
 template <class P, int TY>
 cudaError_t launch_c(int units, cudaStream_t s, const DescC* d, CavityRun* c, int par)
 {
-    const size_t sm = sizeof(SmemC<P, kTileX, TY>);
-    return launch_chained(curv_step_kernel<P, kTileX, TY>, units, kTileX * TY, sm, s, d, c, par);
+    using K = StepC<P, TY>;
+    return launch_chained(K::fn, units, K::threads, K::smem, s, d, c, par);
 }
 
 template <class P, int TY>
 cudaError_t prepare_c()
 {
-    const size_t sm = sizeof(SmemC<P, kTileX, TY>);
-    cudaError_t e = cudaFuncSetAttribute(curv_step_kernel<P, kTileX, TY>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    using K = StepC<P, TY>;
+    cudaError_t e =
+        cudaFuncSetAttribute(K::fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)K::smem);
     if (e != cudaSuccess) return e;
     // the staged geometry makes shared memory the resource that bounds
     // resident blocks: all of the unified L1/shared array to shared memory
-    return cudaFuncSetAttribute(curv_step_kernel<P, kTileX, TY>,
-                                cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    return cudaFuncSetAttribute(K::fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
 }
 
 }  // namespace rtlbfsc
@@ -877,32 +853,37 @@ void append_heat_geo(std::vector<unsigned char>& buf, size_t& off_i, size_t& off
     off_ia = append_array(buf, ia);
 }
 
-// The step kernel's arrays in precision R: face records, the cells'
-// Green-Gauss coefficients (formed in FP64) and dt / area.
-template <typename R>
+// Green-Gauss coefficients of a cell, formed in FP64.
+void cell_grad(int ni, int i, int j, const std::vector<FaceGeo<double>>& fi,
+               const std::vector<FaceGeo<double>>& fj, const std::vector<double>& ia, double k[8])
+{
+    const FaceGeo<double>& fw = fi[(size_t)j * (ni + 1) + i];
+    const FaceGeo<double>& fe = fi[(size_t)j * (ni + 1) + i + 1];
+    const FaceGeo<double>& fs = fj[(size_t)j * ni + i];
+    const FaceGeo<double>& fn = fj[(size_t)(j + 1) * ni + i];
+    const double a = ia[(size_t)j * ni + i];
+    const double we = a * fe.wR, ww = -a * (1.0 - fw.wR);
+    const double wn = a * fn.wR, ws = -a * (1.0 - fs.wR);
+    k[0] = we * fe.Sx, k[1] = we * fe.Sy, k[2] = ww * fw.Sx, k[3] = ww * fw.Sy;
+    k[4] = wn * fn.Sx, k[5] = wn * fn.Sy, k[6] = ws * fs.Sx, k[7] = ws * fs.Sy;
+}
+
+// The FP64 step kernel's arrays: face records, the cells' Green-Gauss
+// coefficients and dt / area.
 void append_step_geo(std::vector<unsigned char>& buf, size_t& off_i, size_t& off_j, size_t& off_cg,
                      size_t& off_dta, int ni, int nj, const std::vector<FaceGeo<double>>& fi,
                      const std::vector<FaceGeo<double>>& fj, const std::vector<double>& ia, double dt)
 {
-    std::vector<FaceRec<R>> ri(fi.size()), rj(fj.size());
-    for (size_t k = 0; k < fi.size(); ++k) ri[k] = face_rec<R>(fi[k]);
-    for (size_t k = 0; k < fj.size(); ++k) rj[k] = face_rec<R>(fj[k]);
-    std::vector<CellGrad<R>> cg((size_t)ni * nj);
-    std::vector<R> dta((size_t)ni * nj);
+    std::vector<FaceRec<double>> ri(fi.size()), rj(fj.size());
+    for (size_t k = 0; k < fi.size(); ++k) ri[k] = face_rec<double>(fi[k]);
+    for (size_t k = 0; k < fj.size(); ++k) rj[k] = face_rec<double>(fj[k]);
+    std::vector<CellGrad<double>> cg((size_t)ni * nj);
+    std::vector<double> dta((size_t)ni * nj);
     for (int j = 0; j < nj; ++j)
         for (int i = 0; i < ni; ++i) {
             const size_t c = (size_t)j * ni + i;
-            const FaceGeo<double>& fw = fi[(size_t)j * (ni + 1) + i];
-            const FaceGeo<double>& fe = fi[(size_t)j * (ni + 1) + i + 1];
-            const FaceGeo<double>& fs = fj[(size_t)j * ni + i];
-            const FaceGeo<double>& fn = fj[(size_t)(j + 1) * ni + i];
-            const double a = ia[c];
-            const double we = a * fe.wR, ww = -a * (1.0 - fw.wR);
-            const double wn = a * fn.wR, ws = -a * (1.0 - fs.wR);
-            const double k[8] = {we * fe.Sx, we * fe.Sy, ww * fw.Sx, ww * fw.Sy,
-                                 wn * fn.Sx, wn * fn.Sy, ws * fs.Sx, ws * fs.Sy};
-            for (int e = 0; e < 8; ++e) cg[c].c[e] = (R)k[e];
-            dta[c] = (R)(dt * a);
+            cell_grad(ni, i, j, fi, fj, ia, cg[c].c);
+            dta[c] = dt * ia[c];
         }
     off_i = append_array(buf, ri);
     off_j = append_array(buf, rj);
@@ -910,11 +891,89 @@ void append_step_geo(std::vector<unsigned char>& buf, size_t& off_i, size_t& off
     off_dta = append_array(buf, dta);
 }
 
+// The FP32 step kernel's arrays in strips (see PairRow), padded with zeros.
+//
+// A wall ghost's gradient is its partner's, sum_f c_f d_f over the
+// differences d_f to the four neighbours, reflected in the face normal: even
+// quantities by M = I - 2 n n^T, odd ones by -M.  A ghost column's
+// differences, over values mirrored two deep, are the partner's times +1 or
+// -1 the same way, with east and west exchanged: its coefficients are M c_f
+// with east and west exchanged, for every quantity.  A ghost row holds M c_f
+// for the partner row's differences; the kernel gives the sign.  A far-field
+// ghost has no gradient.
+void append_pair_geo(std::vector<unsigned char>& buf, size_t& off_i, size_t& off_j, size_t& off_cg,
+                     size_t& off_dta, int rows, const rtlbfsc_ctx* h,
+                     const std::vector<FaceGeo<double>>& fi, const std::vector<FaceGeo<double>>& fj,
+                     const std::vector<double>& ia)
+{
+    const int ni = h->ni, nj = h->nj, X = kPairX, strips = (ni + X - 1) / X;
+    const bool per = h->per != 0;
+    // formed in place: the arrays are the bulk of the upload
+    auto room = [&](size_t bytes) {
+        const size_t o = align256(buf);
+        buf.resize(o + bytes);
+        return o;
+    };
+    off_i = room((size_t)strips * rows * sizeof(PairFaceI));
+    off_j = room((size_t)strips * (rows + 1) * sizeof(PairFaceJ));
+    off_cg = room((size_t)strips * (rows + 2) * sizeof(PairRow));
+    off_dta = room((size_t)strips * rows * X * sizeof(float));
+    PairFaceI* pi = reinterpret_cast<PairFaceI*>(buf.data() + off_i);
+    PairFaceJ* pj = reinterpret_cast<PairFaceJ*>(buf.data() + off_j);
+    PairRow* pc = reinterpret_cast<PairRow*>(buf.data() + off_cg);
+    float* dta = reinterpret_cast<float*>(buf.data() + off_dta);
+    auto put = [](const FaceGeo<double>& f, float* dst, size_t stride) {
+        const FaceRec<float> r = face_rec<float>(f);
+        const float k[12] = {r.nx, r.ny, r.tL, r.tR, r.h, r.cL, r.cR, r.m_nu_2h,
+                             r.m_chi_2h, r.m_tf15, r.m_tg15, r.len};
+        for (int e = 0; e < 12; ++e) dst[e * stride] = k[e];
+    };
+    for (int s = 0; s < strips; ++s) {
+        const int i0 = s * X;
+        for (int j = 0; j < nj; ++j)
+            for (int i = i0; i <= std::min(i0 + X, ni); ++i) {
+                PairFaceI& r = pi[(size_t)s * rows + j];
+                put(fi[(size_t)j * (ni + 1) + i], &r.f[0][i - i0], X + 2);
+                if (i < std::min(i0 + X, ni))
+                    dta[((size_t)s * rows + j) * X + i - i0] = (float)(h->dt * ia[(size_t)j * ni + i]);
+            }
+        for (int j = 0; j <= nj; ++j)
+            for (int i = i0; i < std::min(i0 + X, ni); ++i)
+                put(fj[(size_t)j * ni + i], &pj[(size_t)s * (rows + 1) + j].f[0][i - i0], X);
+        for (int j = -1; j <= nj; ++j)
+            for (int i = i0 - 1; i <= i0 + X; ++i) {
+                int is, xs, js, ys;
+                const bool in = resolve_c(i, ni, per, 0, 1, is, xs);
+                resolve_c(j, nj, false, 2, 3, js, ys);
+                const int side = xs >= 0 ? xs : ys;
+                if (!in || (xs >= 0 && ys >= 0) || (side >= 0 && h->kind[side] == kFar)) continue;
+                double k[8];
+                cell_grad(ni, is, js, fi, fj, ia, k);
+                if (side >= 0) {  // the boundary face of the partner
+                    const FaceGeo<double>& fb = xs >= 0 ? fi[(size_t)js * (ni + 1) + (xs ? ni : 0)]
+                                                        : fj[(size_t)(ys == 3 ? nj : 0) * ni + is];
+                    for (int f = 0; f < 4; ++f) {
+                        const double n = k[2 * f] * fb.nx + k[2 * f + 1] * fb.ny;
+                        k[2 * f] -= 2.0 * n * fb.nx;
+                        k[2 * f + 1] -= 2.0 * n * fb.ny;
+                    }
+                }
+                if (xs >= 0) {
+                    std::swap(k[0], k[2]);
+                    std::swap(k[1], k[3]);
+                }
+                for (int e = 0; e < 8; ++e)
+                    pc[(size_t)s * (rows + 2) + j + 1].c[e][i - i0 + 2] = (float)k[e];
+            }
+    }
+}
+
 int tile_rows_of(const rtlbfsc_ctx* h)
 {
     if (h->tile_rows == 8 || h->tile_rows == 16) return h->tile_rows;
     // 32 x 8 by default: four resident blocks per SM against two of the
-    // 32 x 16 tile (measured faster on small and large O-meshes alike)
+    // 32 x 16 tile (FP32 at 150 x 100: 5.5 us against 6.4, at 1800 x 1200: 123
+    // against 133)
     return 8;
 }
 
@@ -938,11 +997,14 @@ int upload(rtlbfsc_ctx* h)
         for (int i = 0; i < ni; ++i) ia[(size_t)j * ni + i] = 1.0 / g.area[g.id(i, j)];
     std::vector<unsigned char> buf;
     size_t oi_d, oj_d, oia_d, oi, oj, ocg, odta;
+    const int pair_rows = (nj + 15) / 16 * 16;  // whole tiles of either height
+    // one allocation: the FP64 arrays and at most as much again
+    buf.reserve(2 * (fi.size() + fj.size()) * sizeof(FaceGeo<double>) + 16 * ia.size() + (1u << 20));
     append_heat_geo(buf, oi_d, oj_d, oia_d, fi, fj, ia);
     if (h->precision == RTLBFS_FP64)
-        append_step_geo<double>(buf, oi, oj, ocg, odta, ni, nj, fi, fj, ia, h->dt);
+        append_step_geo(buf, oi, oj, ocg, odta, ni, nj, fi, fj, ia, h->dt);
     else
-        append_step_geo<float>(buf, oi, oj, ocg, odta, ni, nj, fi, fj, ia, h->dt);
+        append_pair_geo(buf, oi, oj, ocg, odta, pair_rows, h, fi, fj, ia);
     if (h->d_geo) {
         cudaStreamSynchronize(h->stream);
         cudaFree(h->d_geo);
@@ -955,6 +1017,7 @@ int upload(rtlbfsc_ctx* h)
     d.ni = ni;
     d.nj = nj;
     d.per = h->per;
+    d.pair_rows = pair_rows;
     const int ty = tile_rows_of(h);
     d.tiles_x = (ni + kTileX - 1) / kTileX;
     d.tiles_y = (nj + ty - 1) / ty;
