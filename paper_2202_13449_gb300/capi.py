@@ -795,7 +795,8 @@ class Solver3:
 
     def set_schedule(self, tile: int = 0, kchunk: int = 0):
         """tile 0: 32 x 4, 1: 16 x 8, 2: 32 x 8 columns per block; kchunk
-        z-planes per work unit (0: automatic)."""
+        z-planes per work unit (0: automatic).  A solver that was neither
+        scheduled nor tuned picks its tile by size."""
         self._check(lib().rtlbfs3d_set_schedule(self._h, int(tile), int(kchunk)), "set_schedule")
 
     def autotune(self, steps: int = 32):

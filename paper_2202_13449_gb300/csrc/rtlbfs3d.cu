@@ -815,6 +815,7 @@ struct rtlbfs3d_ctx {
     double bcT[6] = {0.0, 1.0, 0.0, 0.0, 0.0, 0.0};
     double bcU[6][3] = {};
     int tile = 0, kchunk_req = 0;
+    bool auto_tile = true;  // until a schedule is set or timed
     int scheme = 0;  // face stage: 0 RTLBFS (Section 3.2), 1 TLBFS (Section 2.2)
     int sms = 0, occ[3][2] = {};
     // device memory
@@ -887,42 +888,66 @@ int resolve(rtlbfs3d_ctx* h)
     return RTLBFS_OK;
 }
 
-// units of the current schedule
+// Modelled time of a step, in us, and the chunk of the least.
+//
+// A unit takes its planes, at `plane` us each when alone on its SM, and the
+// like of `extra` more for the planes below it; units on an SM at once slow
+// each other by `slow` per unit beyond the first: in FP32 by 8 % a warp
+// (latency hides in the others' gaps), in FP64 by the share of the FP64 units
+// each needs.  80^3 in 16 x 8 tiles, time over that of the pick, modelled and
+// measured: FP32 (pick 7 planes, 48 us) 4 planes 1.22 and 1.26, 8 planes 1.11
+// and 1.11; FP64 (pick 9, 1336 us) 4 planes 1.15 and 1.16, 8 planes 1.27 and
+// 1.14.  Where the mesh leaves SMs idle the pick is a plane or two: 16^3 12 us
+// (FP64 92), against 22 (269) with chunks of 4.
+double model_step(const rtlbfs3d_ctx* h, int tile, int& kc)
+{
+    const int TX = kTiles[tile][0], TY = kTiles[tile][1];
+    const bool fp64 = h->precision == RTLBFS_FP64;
+    const int occ = std::max(1, h->occ[tile][h->scheme]), sms = std::max(1, h->sms);
+    const long long per_plane =
+        (long long)((h->n[0] + TX - 1) / TX) * ((h->n[1] + TY - 1) / TY);
+    const double warps = TX * TY / (fp64 ? 32 : 64), extra = fp64 ? 0.55 : 1.5;
+    const double slow = fp64 ? 0.35 + 0.0875 * warps : 0.08 * warps;
+    const double plane = fp64 ? (tile == 2 ? 85.0 : 60.0) : (tile == 2 ? 4.1 : 3.6);
+    auto busy = [&](long long m) { return m > 0 ? 1.0 + slow * (m - 1) : 0.0; };
+    auto time = [&](int k) {
+        const long long units = per_plane * ((h->n[2] + k - 1) / k);
+        const long long b = (units + sms - 1) / sms;  // units of the busiest SM
+        return plane * (k + extra) * ((b / occ) * busy(occ) + busy(b % occ));
+    };
+    if (h->kchunk_req > 0) {
+        kc = std::min(h->kchunk_req, h->n[2]);
+        return time(kc);
+    }
+    double best = INFINITY;
+    for (int k = 1; k <= h->n[2]; ++k)
+        if (time(k) < best) {
+            best = time(k);
+            kc = k;
+        }
+    return best;
+}
+
+// units of the current schedule; the tile of the least modelled time unless
+// one was chosen.  FP32, 32 x 4, 16 x 8 and 32 x 8 at 48^3: 20.8, 19.7 and
+// 21.0 us; at 80^3 53.6, 48.4 and 54.6; at 160^3 310, 313 and 279 (modelled
+// order the same; 16 x 8 is preferred where they tie).
 void decompose(rtlbfs3d_ctx* h, Desc3& d)
 {
+    int kc = 1;
+    double best = INFINITY;
+    if (h->auto_tile)
+        for (int t : {1, 0, 2}) {
+            const double us = model_step(h, t, kc);
+            if (us < best) {
+                best = us;
+                h->tile = t;
+            }
+        }
+    model_step(h, h->tile, kc);
     const int TX = kTiles[h->tile][0], TY = kTiles[h->tile][1];
     d.tiles_x = (h->n[0] + TX - 1) / TX;
     d.tiles_y = (h->n[1] + TY - 1) / TY;
-    int kc = h->kchunk_req;
-    if (kc <= 0) {
-        // The chunk of the least modelled time.  A unit takes its planes and
-        // the like of `extra` more for the planes below it; units on an SM at
-        // once slow each other by `slow` per unit beyond the first: in FP32
-        // by 8 % a warp (latency hides in the others' gaps), in FP64 by the
-        // share of the FP64 units each needs.  80^3 in 16 x 8 tiles, time
-        // over that of the pick, modelled and measured: FP32 (pick 7 planes,
-        // 48 us) 4 planes 1.22 and 1.26, 8 planes 1.11 and 1.11; FP64 (pick
-        // 9, 1336 us) 4 planes 1.15 and 1.16, 8 planes 1.27 and 1.14.  Where
-        // the mesh leaves SMs idle the pick is a plane or two: 16^3 12 us
-        // (FP64 92), against 22 (269) with chunks of 4.
-        const bool fp64 = h->precision == RTLBFS_FP64;
-        const int occ = std::max(1, h->occ[h->tile][h->scheme]), sms = std::max(1, h->sms);
-        const long long per_plane = (long long)d.tiles_x * d.tiles_y;
-        const double warps = TX * TY / (fp64 ? 32 : 64), extra = fp64 ? 0.55 : 1.5;
-        const double slow = fp64 ? 0.35 + 0.0875 * warps : 0.08 * warps;
-        auto busy = [&](long long m) { return m > 0 ? 1.0 + slow * (m - 1) : 0.0; };
-        double best = INFINITY;
-        for (int k = 1; k <= h->n[2]; ++k) {
-            const long long units = per_plane * ((h->n[2] + k - 1) / k);
-            const long long b = (units + sms - 1) / sms;  // units of the busiest SM
-            const double t = (k + extra) * ((b / occ) * busy(occ) + busy(b % occ));
-            if (t < best) {
-                best = t;
-                kc = k;
-            }
-        }
-    }
-    kc = std::min(kc, h->n[2]);
     d.kchunk = kc;
     d.chunks = (h->n[2] + kc - 1) / kc;
     d.units = d.tiles_x * d.tiles_y * d.chunks;
@@ -1519,6 +1544,7 @@ int rtlbfs3d_set_schedule(rtlbfs3d_t h, int tile, int kchunk)
     if (bad_handle(h)) return RTLBFS_ERR_ARG;
     if (tile < 0 || tile > 2 || kchunk < 0) return h->fail(RTLBFS_ERR_ARG, "bad schedule");
     h->tile = tile;
+    h->auto_tile = false;
     h->kchunk_req = kchunk;
     h->dirty = true;
     return RTLBFS_OK;
@@ -1545,6 +1571,8 @@ int rtlbfs3d_autotune(rtlbfs3d_t h, int steps, int* tile, double* ms_per_step)
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
     const int keep_k = h->kchunk_req;
+    const bool keep_auto = h->auto_tile;
+    h->auto_tile = false;
     int best = h->tile;
     float best_ms = INFINITY;
     for (int t = 0; t < 3 && rc == RTLBFS_OK; ++t) {
@@ -1578,7 +1606,11 @@ int rtlbfs3d_autotune(rtlbfs3d_t h, int steps, int* tile, double* ms_per_step)
         const int prc = put_run(h, saved);
         if (!rc) rc = prc;
     }
-    if (rc) return rc;
+    if (rc) {
+        h->auto_tile = keep_auto;
+        h->dirty = true;
+        return rc;
+    }
     h->tile = best;
     h->dirty = true;
     rc = upload(h);
