@@ -198,11 +198,18 @@ WORKLOADS = {
 DEFAULT_WORKLOAD = "cavity512"
 STEP3_SOURCES = ["paper_2202_13449_gb300/csrc/rtlbfs3d.cu",
                  "paper_2202_13449_gb300/csrc/rtlbfs3d_dev.cuh",
+                 "paper_2202_13449_gb300/csrc/rtlbfs3d_pair.cuh",
+                 "paper_2202_13449_gb300/csrc/rtlbfs_pair.cuh",
                  "paper_2202_13449_gb300/csrc/rtlbfs_dev.cuh"]
 CURV_SOURCES = ["paper_2202_13449_gb300/csrc/rtlbfs_curv.cu",
+                "paper_2202_13449_gb300/csrc/rtlbfs_curv_pair.cuh",
+                "paper_2202_13449_gb300/csrc/rtlbfs_pair.cuh",
                 "paper_2202_13449_gb300/csrc/rtlbfs_dev.cuh"]
 STEP_SOURCES = ["paper_2202_13449_gb300/csrc/rtlbfs_step.cu",
                 "paper_2202_13449_gb300/csrc/rtlbfs_march.cu",
+                "paper_2202_13449_gb300/csrc/rtlbfs_march2.cu",
+                "paper_2202_13449_gb300/csrc/rtlbfs_pair.cuh",
+                "paper_2202_13449_gb300/csrc/rtlbfs_tile_pair.cuh",
                 "paper_2202_13449_gb300/csrc/rtlbfs_dev.cuh",
                 "paper_2202_13449_gb300/csrc/rtlbfs_kernels.h",
                 "paper_2202_13449_gb300/csrc/rtlbfs_tile.cuh",
@@ -210,6 +217,11 @@ STEP_SOURCES = ["paper_2202_13449_gb300/csrc/rtlbfs_step.cu",
 # schedule kernel kinds of the 2D solver: short names and device kernel names
 SCHED_NAMES = ["march", "tile", "persist"]
 SCHED_KERNELS = ["rtlbfs::march_kernel", "rtlbfs::step_kernel", "rtlbfs::persist_kernel"]
+
+
+def sched_kernel(kind: int, real_bytes: int) -> str:
+    """Device kernel of a schedule kind: marching in FP32 is march2_kernel."""
+    return "rtlbfs::march2_kernel" if kind == 0 and real_bytes == 4 else SCHED_KERNELS[kind]
 
 
 def kernel_hash(sources=None) -> str:
@@ -480,7 +492,7 @@ def run_batch(args, w):
     value = cells * inner * args.steps * ws / (ms * 1e-3) / 1e6
     rs = 4 if prec == capi.FP32 else 8
     per_launch = ms * 1e-3 / (inner * args.steps)
-    kname = SCHED_KERNELS[sched[0]]
+    kname = sched_kernel(sched[0], rs)
     traffic = profile_traffic(args.workload, w["precision"], SCHED_NAMES[sched[0]])
     alu, hbm = rooflines(kname, cells, per_launch, rs, traffic, clocks)
 
@@ -1043,12 +1055,12 @@ def run_cubic(args, w):
         "gpu_launches": int(launches),
         "roofline": {"bound": "alu", "achieved": round(alu, 3), "peak": round(peak_alu, 3),
                      "unit": unit, "frac": round(alu / peak_alu, 4), "traffic": traffic,
-                     "kernel": "rtlbfs3::step3_kernel", "ops_per_cell_update": ops_cell,
+                     "kernel": "rtlbfs3::step3_pair_kernel" if rs == 4 else "rtlbfs3::step3_kernel", "ops_per_cell_update": ops_cell,
                      "sfu_ops_per_cell_update": sfu_cell, "peak_source": src,
                      "alg_ops_per_launch": ops_cell * cells},
         "roofline_hbm": {"bound": "hbm", "achieved": round(hbm, 1), "peak": peak, "unit": "GB/s",
                          "frac": round(hbm / peak, 4), "traffic": traffic,
-                         "kernel": "rtlbfs3::step3_kernel",
+                         "kernel": "rtlbfs3::step3_pair_kernel" if rs == 4 else "rtlbfs3::step3_kernel",
                          "peak_source": f"{peak_kind} hbm_gbs", "alg_bytes_per_launch": alg_bytes},
         "table6_context": {"steps_for_t_star_1": steps_t1,
                            "device_s_for_t_star_1": round(steps_t1 * per_launch_s, 3),
@@ -1543,7 +1555,7 @@ def run_curv(args, w):
         "roofline": {"bound": "alu", "achieved": round(alu, 3), "peak": round(peak_alu, 3),
                      "unit": "T FP32 op/s" if rs == 4 else "T FP64 op/s",
                      "frac": round(alu / peak_alu, 4), "traffic": traffic,
-                     "kernel": "rtlbfsc::curv_step_kernel", "ops_per_cell_update": ops_cell,
+                     "kernel": "rtlbfsc::curv_pair_kernel" if rs == 4 else "rtlbfsc::curv_step_kernel", "ops_per_cell_update": ops_cell,
                      "sfu_ops_per_cell_update": sfu_cell, "peak_source": src},
         "roofline_hbm": {"bound": "hbm", "achieved": round(alg_bytes / per_launch / 1e9, 1),
                          "peak": peak, "unit": "GB/s",
@@ -1688,7 +1700,7 @@ def run_ours(args, w):
 
     rs = 4 if w["precision"] == "fp32" else 8
     per_launch_s = ms_max * 1e-3 / (inner * args.steps)
-    kname = SCHED_KERNELS[sched[0]]
+    kname = sched_kernel(sched[0], rs)
     traffic = profile_traffic(args.workload, w["precision"], SCHED_NAMES[sched[0]])
     alu, hbm = rooflines(kname, cells, per_launch_s, rs, traffic, clocks, w.get("scheme", 0))
     res, steps_total = s.residual()
@@ -1817,7 +1829,7 @@ def run_strips(args, w):
     e2e = nx * ny * inner * 2 / job_max(time.perf_counter() - t0) / 1e6
     assert np.all(np.isfinite(out[3]))
     per_step_s = ms_max * 1e-3 / (inner * args.steps)
-    kname = SCHED_KERNELS[sched[0]] if sched else "rtlbfs::march_kernel"
+    kname = sched_kernel(sched[0] if sched else 0, 4)
     alu, hbm = rooflines(kname, cells_mine, per_step_s, 4, None, clocks)
     line = {
         "metric": "M cell-updates/s (whole job) and fraction of the ALU and HBM rooflines",

@@ -8,7 +8,7 @@
 // 48 us a step; a thread per cell in scalar arithmetic took 67, issue-bound at
 // 3250 instructions a cell.  What bounds it now is latency: 1500 instructions
 // a cell keep the schedulers busy a third of the time with the 8 warps that
-// 230 registers a thread leave room for (128^3 in 32 x 8: 55 % with 12).
+// 230 registers a thread leave room for (large meshes in 32 x 8: half of it with 12).
 //  - Face fluxes change hands as registers (x: shuffles) or through shared
 //    memory (y, and the tile's east column), so that three 32 x 8 blocks fit.
 //  - Raw records of the plane to come are fetched after the faces, which need

@@ -19,10 +19,10 @@
 // Why two columns a lane: the step is bound by instruction issue and the FMA
 // pipe.  A packed instruction does two columns' operation in one issue slot;
 // only one of a pair's two x-neighbours needs a shuffle; 4 of 64 columns are
-// halo instead of 4 of 32.  Per cell 406 thread instructions instead of the
-// 727 of a scalar march with one column a lane; the FMA pipe is the bound
-// (a packed FMA holds it for two cycles), about 70 % busy at 4096^2: 476 ->
-// 351 us per step there (35 -> 48 G cell-updates/s), 1024^2 42 -> 36 us.
+// halo instead of 4 of 32.  Per cell 444 thread instructions instead of the
+// 727 of a scalar march with one column a lane; the FMA pipe leads (a packed
+// FMA holds it for two cycles), 61 % busy at 4096^2: 476 -> 336 us per step
+// there (35 -> 50 G cell-updates/s), 1024^2 42 -> 33.5 us.
 // One warp a block: twelve fit an SM without spills (168 registers), where
 // blocks of four warps compile to 220 registers and eight warps.
 // A row's raw records come by asynchronous copies into a ring in shared

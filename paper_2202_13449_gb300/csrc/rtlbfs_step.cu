@@ -13,9 +13,10 @@
 //      (Eqs. 46-48), corrector fluxes (Eqs. 57-59) -- face_flux();
 //   4. the explicit update with the Boussinesq source (Eq. 64) and the
 //      conservative -> primitive conversion;
-//   5. the residual sums of the steady criterion; the last tile of a cavity
-//      to finish turns them into (R_u, R_T), advances the step counter,
-//      flips the buffer and decides whether the cavity is done.
+//   5. the residual sums of the steady criterion; the next launch turns them
+//      into (R_u, R_T), advances the step counter, flips the buffer and
+//      decides whether the cavity is done.
+// FP32 tiles do this in pairs of columns (rtlbfs_tile_pair.cuh).
 // Face values and gradients never leave the SM; HBM sees one read and one
 // write of the four fields per cell per step (halo re-reads hit L2).
 #include <cuda_runtime.h>

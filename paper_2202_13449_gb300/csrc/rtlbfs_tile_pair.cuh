@@ -3,8 +3,8 @@
 //
 // A small mesh's step is one block's chain of loads, phases and barriers; a
 // large one's is the instructions of all.  Against one column at a time:
-//   - the arithmetic of two columns in one instruction (605 thread
-//     instructions per cell-update, load and overheads included, were 809);
+//   - the arithmetic of two columns in one instruction (588 thread
+//     instructions per cell-update at 512^2, overheads included, were 829);
 //   - a warp evaluates one x- or y-face pair where the mesh leaves an SM one
 //     tile (four times the warps a block), two or four elsewhere;
 //   - ghost columns hold mirrored values two deep, so gradients need no rule
