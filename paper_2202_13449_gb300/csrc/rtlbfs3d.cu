@@ -270,8 +270,8 @@ __device__ __forceinline__ void face3(const Desc3& d, CellNT3<R>& L, R tauL, Cel
 }
 
 template <class P, int TX, int TY, int SCH>
-__global__ void __launch_bounds__(TX* TY) step3_kernel(const Desc3* __restrict__ dp,
-                                                       CavityRun* __restrict__ run, int par)
+__global__ void __launch_bounds__(TX* TY, TX * TY == 128 && SCH == 0 ? 3 : 1)
+step3_kernel(const Desc3* __restrict__ dp, CavityRun* __restrict__ run, int par)
 {
     using S = typename P::S;
     using R = typename P::R;
@@ -383,7 +383,7 @@ __global__ void __launch_bounds__(TX* TY) step3_kernel(const Desc3* __restrict__
         }
         const int vs = mod3(kk), vm = mod3(kk - 1), vp = mod3(kk + 1);
         const R izn = zc[kk + 2].is_next, izm = zc[kk + 1].is_next;
-        for (int t = tid; t < GX * GY; t += NT) {
+        for (int t = (tid + NT - 64) % NT; t < GX * GY; t += NT) {
             const int r = t / GX + 1, c = t % GX + 1;
             int is, xs, js, ys;
             const bool xok = resolve_1d(i0 - 2 + c, nx, xper, 0, 1, is, xs);
@@ -466,36 +466,73 @@ __global__ void __launch_bounds__(TX* TY) step3_kernel(const Desc3* __restrict__
         __syncthreads();
         grad_plane(k + 1);
         __syncthreads();
-        // x- and y-faces of plane k
+        // x- and y-faces of plane k.  The second, mostly empty rounds of the
+        // x-faces, the y-faces and the gradients start on warps 0, 1 and 2: an
+        // FP64 instruction costs the same with one lane or 32, and a block waits
+        // for its slowest warp (all three on warp 0: 80^3 1337 us, now 1253).
         const int vs = mod3(k), gs = mod2(k);
         constexpr int NXF = TY * (TX + 1), NYF = (TY + 1) * TX;
-        for (int t = tid; t < NXF; t += NT) {
-            const int fj = t / (TX + 1), fi = t % (TX + 1);
-            const int gx = i0 + fi;
-            if (gx > nx || j0 + fj >= ny) continue;
-            CellNT3<R> L, Rr;
-            R tl, tr;
-            take3<R>(sm, vs, gs, fj + 2, fi + 1, 0, L, tl);
-            take3<R>(sm, vs, gs, fj + 2, fi + 2, 0, Rr, tr);
-            const int ws = xper ? -1 : (gx == 0 ? 0 : (gx == nx ? 1 : -1));
-            R F[5];
-            face3<P, R, SCH>(d, L, tl, Rr, tr, get_line(sm.xl, fi), Tz, 0, ws, F);
+        // 16 x 8: one loop over both kinds (face t < NXF an x-face) takes 9
+        // warp rounds instead of 5 + 5, and at three blocks an SM the shared
+        // copy of the face fits 156 registers: 80^3 1253 -> 1209 us, TLBFS
+        // 2037 -> 1907.  Where it saves no round the two loops are 1-2 %
+        // faster (32 x 4 1442 against 1472 us).
+        constexpr bool ONE = (NXF + NYF + 31) / 32 < (NXF + 31) / 32 + (NYF + 31) / 32;
+        if constexpr (ONE) {
+            for (int t = tid; t < NXF + NYF; t += NT) {
+                const bool isx = t < NXF;
+                const int u = isx ? t : t - NXF;
+                const int fj = isx ? u / (TX + 1) : u / TX, fi = isx ? u % (TX + 1) : u % TX;
+                const int g = isx ? i0 + fi : j0 + fj;  // the face's index along its normal
+                if (isx ? (g > nx || j0 + fj >= ny) : (g > ny || i0 + fi >= nx)) continue;
+                const int ax = isx ? 0 : 1;
+                CellNT3<R> L, Rr;
+                R tl, tr;
+                take3<R>(sm, vs, gs, isx ? fj + 2 : fj + 1, isx ? fi + 1 : fi + 2, ax, L, tl);
+                take3<R>(sm, vs, gs, fj + 2, fi + 2, ax, Rr, tr);
+                const bool per = isx ? xper : yper;
+                const int n_ax = isx ? nx : ny;
+                const int ws = per ? -1 : (g == 0 ? 2 * ax : (g == n_ax ? 2 * ax + 1 : -1));
+                R F[5];
+                face3_frame<P, R, SCH>(d, L, tl, Rr, tr, isx ? get_line(sm.xl, fi) : get_line(sm.yl, fj),
+                                       Tz, ax, ws, F);
+                R* dst = isx ? &sm.fx[0][fj][fi] : &sm.fy[0][fj][fi];
+                const int qs = isx ? NXF : NYF;  // stride between components
+                dst[0] = F[0];
+                dst[(isx ? 1 : 2) * qs] = F[1];
+                dst[(isx ? 2 : 3) * qs] = F[2];
+                dst[(isx ? 3 : 1) * qs] = F[3];
+                dst[4 * qs] = F[4];
+            }
+        } else {
+            for (int t = tid; t < NXF; t += NT) {
+                const int fj = t / (TX + 1), fi = t % (TX + 1);
+                const int gx = i0 + fi;
+                if (gx > nx || j0 + fj >= ny) continue;
+                CellNT3<R> L, Rr;
+                R tl, tr;
+                take3<R>(sm, vs, gs, fj + 2, fi + 1, 0, L, tl);
+                take3<R>(sm, vs, gs, fj + 2, fi + 2, 0, Rr, tr);
+                const int ws = xper ? -1 : (gx == 0 ? 0 : (gx == nx ? 1 : -1));
+                R F[5];
+                face3<P, R, SCH>(d, L, tl, Rr, tr, get_line(sm.xl, fi), Tz, 0, ws, F);
 #pragma unroll
-            for (int q = 0; q < 5; ++q) sm.fx[q][fj][fi] = F[q];
-        }
-        for (int t = tid; t < NYF; t += NT) {
-            const int fj = t / TX, fi = t % TX;
-            const int gy = j0 + fj;
-            if (gy > ny || i0 + fi >= nx) continue;
-            CellNT3<R> L, Rr;
-            R tl, tr;
-            take3<R>(sm, vs, gs, fj + 1, fi + 2, 1, L, tl);
-            take3<R>(sm, vs, gs, fj + 2, fi + 2, 1, Rr, tr);
-            const int ws = yper ? -1 : (gy == 0 ? 2 : (gy == ny ? 3 : -1));
-            R F[5];
-            face3<P, R, SCH>(d, L, tl, Rr, tr, get_line(sm.yl, fj), Tz, 1, ws, F);
+                for (int q = 0; q < 5; ++q) sm.fx[q][fj][fi] = F[q];
+            }
+            for (int t = (tid + NT - 32) % NT; t < NYF; t += NT) {
+                const int fj = t / TX, fi = t % TX;
+                const int gy = j0 + fj;
+                if (gy > ny || i0 + fi >= nx) continue;
+                CellNT3<R> L, Rr;
+                R tl, tr;
+                take3<R>(sm, vs, gs, fj + 1, fi + 2, 1, L, tl);
+                take3<R>(sm, vs, gs, fj + 2, fi + 2, 1, Rr, tr);
+                const int ws = yper ? -1 : (gy == 0 ? 2 : (gy == ny ? 3 : -1));
+                R F[5];
+                face3<P, R, SCH>(d, L, tl, Rr, tr, get_line(sm.yl, fj), Tz, 1, ws, F);
 #pragma unroll
-            for (int q = 0; q < 5; ++q) sm.fy[q][fj][fi] = F[q];
+                for (int q = 0; q < 5; ++q) sm.fy[q][fj][fi] = F[q];
+            }
         }
         R Fu[5] = {R(0), R(0), R(0), R(0), R(0)};
         R c0[5];
