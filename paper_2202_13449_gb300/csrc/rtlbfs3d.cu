@@ -269,8 +269,9 @@ __device__ __forceinline__ void face3(const Desc3& d, CellNT3<R>& L, R tauL, Cel
     out[4] = F[4];
 }
 
+// (resident blocks as shared memory allows: registers up to 255 a thread)
 template <class P, int TX, int TY, int SCH>
-__global__ void __launch_bounds__(TX* TY, TX * TY == 128 && SCH == 0 ? 3 : 1)
+__global__ void __launch_bounds__(TX* TY, TX * TY == 128 ? 2 : 1)
 step3_kernel(const Desc3* __restrict__ dp, CavityRun* __restrict__ run, int par)
 {
     using S = typename P::S;
@@ -473,10 +474,9 @@ step3_kernel(const Desc3* __restrict__ dp, CavityRun* __restrict__ run, int par)
         const int vs = mod3(k), gs = mod2(k);
         constexpr int NXF = TY * (TX + 1), NYF = (TY + 1) * TX;
         // 16 x 8: one loop over both kinds (face t < NXF an x-face) takes 9
-        // warp rounds instead of 5 + 5, and at three blocks an SM the shared
-        // copy of the face fits 156 registers: 80^3 1253 -> 1209 us, TLBFS
-        // 2037 -> 1907.  Where it saves no round the two loops are 1-2 %
-        // faster (32 x 4 1442 against 1472 us).
+        // warp rounds instead of 5 + 5: 80^3 1253 -> 1199 us, TLBFS 2037 ->
+        // 1903.  Where it saves no round the two loops are 1-2 % faster
+        // (32 x 4 1442 against 1472 us).
         constexpr bool ONE = (NXF + NYF + 31) / 32 < (NXF + 31) / 32 + (NYF + 31) / 32;
         if constexpr (ONE) {
             for (int t = tid; t < NXF + NYF; t += NT) {
@@ -933,9 +933,9 @@ int resolve(rtlbfs3d_ctx* h)
 // (latency hides in the others' gaps), in FP64 by the share of the FP64 units
 // each needs.  80^3 in 16 x 8 tiles, time over that of the pick, modelled and
 // measured: FP32 (pick 7 planes, 48 us) 4 planes 1.22 and 1.26, 8 planes 1.11
-// and 1.11; FP64 (pick 9, 1336 us) 4 planes 1.15 and 1.16, 8 planes 1.27 and
-// 1.14.  Where the mesh leaves SMs idle the pick is a plane or two: 16^3 12 us
-// (FP64 92), against 22 (269) with chunks of 4.
+// and 1.11; FP64 (pick 14, 1206 us) 4 planes 1.13 and 1.09, 8 planes 1.18 and
+// 1.15.  Where the mesh leaves SMs idle the pick is a plane or two: 16^3 12 us
+// (FP64 83), against 22 (236) with chunks of 4.
 double model_step(const rtlbfs3d_ctx* h, int tile, int& kc)
 {
     const int TX = kTiles[tile][0], TY = kTiles[tile][1];
