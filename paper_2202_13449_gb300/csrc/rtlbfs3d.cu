@@ -38,6 +38,7 @@
 #include "rtlbfs_dev.cuh"
 #include "rtlbfs_kernels.h"
 #include "rtlbfs_pair.cuh"
+#include "rtlbfs_smem.h"
 
 namespace rtlbfs {
 extern std::atomic<long long> g_launches;
@@ -795,17 +796,17 @@ struct Step3<StoreQ, TX, TY, SCH> {
     static constexpr size_t smem = sizeof(Smem3P<TX, TY>);
 };
 
-// Blocks per SM are held at what one even round of the units needs, by asking
-// for the least shared memory that b + 1 blocks do not find: the blocks of the next step, launched while this one
-// drains, otherwise crowd onto the SMs that empty first. 64^3
-// in 32 x 8 tiles (256 units on 152 SMs): 32 us, 40 without.
+// Blocks per SM are held at what one even round of the units needs
+// (smem_for_blocks): the blocks of the next step, launched while this one
+// drains, otherwise crowd onto the SMs that empty first. 64^3 in 32 x 8 tiles
+// (256 units on 152 SMs): 32 us, 40 without.
 template <class K>
 cudaError_t launch_kernel3(int units, int sms, cudaStream_t s, const Desc3* d, CavityRun* c,
                            int par)
 {
-    const size_t b = (size_t)(units + sms - 1) / sms;
-    const size_t smem = std::max(K::smem, (228 * 1024 / (b + 1) - 1024) / 128 * 128 + 128);
-    return launch_chained(K::fn, units, K::threads, smem, s, d, c, par);
+    const long long b = ((long long)units + sms - 1) / sms;
+    return launch_chained(K::fn, units, K::threads, rtlbfs::smem_for_blocks(K::smem, b), s, d, c,
+                          par);
 }
 
 template <class P, int TX, int TY>
@@ -820,7 +821,7 @@ template <class K>
 cudaError_t prepare_kernel3(int* occ)
 {
     cudaError_t e =
-        cudaFuncSetAttribute(K::fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+        cudaFuncSetAttribute(K::fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rtlbfs::kSmemMax);
     if (e == cudaSuccess)
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, K::fn, K::threads, K::smem);
     return e;

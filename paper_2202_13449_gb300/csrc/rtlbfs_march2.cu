@@ -39,6 +39,7 @@
 #include "rtlbfs_dev.cuh"
 #include "rtlbfs_kernels.h"
 #include "rtlbfs_pair.cuh"
+#include "rtlbfs_smem.h"
 
 namespace rtlbfs {
 
@@ -331,10 +332,6 @@ march2_kernel(const CavityDesc* __restrict__ descs, CavityRun* __restrict__ runs
 }
 
 static constexpr size_t kSmem2 = sizeof(WarpSmem) * (kMarch2Threads / 32);
-
-// An SM's shared memory, what the system takes of it per block, and the most
-// a block may ask for.
-static constexpr size_t kSmemSM = 228 * 1024, kSmemSystem = 1024, kSmemMax = 227 * 1024;
 
 cudaError_t march2_prepare()
 {
