@@ -302,34 +302,6 @@ struct alignas(4 * sizeof(R)) Vec4 {
 template <typename R>
 __host__ __device__ __forceinline__ R rconst(double v) { return static_cast<R>(v); }
 
-// FP64 reciprocal and square root to an ulp or so, from the hardware's
-// approximations: FP64 operations are what the FP64 kernels wait for (an SM
-// does two lanes of one a clock), and the compiler's IEEE-rounded division
-// and root spend more of them on rounding and special cases that the last
-// bit of a reciprocal does not need here.
-//
-// Third-order Newton step: with e = 1 - x r, 1/x = r / (1 - e) = r (1 + e +
-// e^2 + ...), so r + r (e + e^2) is off by e^3 (r good to 2^-20 or better).
-__device__ __forceinline__ double rcp64(double x)
-{
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-    const double e = fma(-x, r, 1.0);
-    return fma(r, fma(e, e, e), r);
-}
-// Newton for y = 1/sqrt(x), then g = x y corrected by its residual (x >= 0;
-// 0 where x underflows the approximation).
-__device__ __forceinline__ double sqrt64(double x)
-{
-    double y;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double g0 = x * y, h0 = 0.5 * y;
-    const double r = fma(-g0, h0, 0.5);
-    const double g = fma(g0, r, g0), h = fma(h0, r, h0);
-    const double s = fma(fma(-g, g, x), h, g);
-    return (unsigned)__double2hiint(x) < 0x00100000u ? 0.0 : s;
-}
-
 // -------------------------------------------------------------------------
 // Value types of the face arithmetic.  float / double: one face.  f2: two
 // faces at once in the packed FP32x2 instructions of sm_100+ (one issue
@@ -363,14 +335,7 @@ struct vtraits<float> {
 template <>
 struct vtraits<double> {
     static __device__ __forceinline__ double bc(double c) { return c; }
-    static __host__ __device__ __forceinline__ double rcp(double x)
-    {
-#ifdef __CUDA_ARCH__
-        return rcp64(x);
-#else
-        return 1.0 / x;
-#endif
-    }
+    static __host__ __device__ __forceinline__ double rcp(double x) { return 1.0 / x; }
     static __host__ __device__ __forceinline__ double neg(double x) { return -x; }
 };
 template <>
@@ -698,8 +663,10 @@ struct StoreD {
     {
         return (__double2hiint(v) & 0x7fffffff) < 0x7ff80000;
     }
-    static __device__ __forceinline__ R rcp(R x) { return rcp64(x); }
-    static __device__ __forceinline__ R fsqrt(R x) { return sqrt64(x); }
+    // IEEE-rounded, with their infinities: a speed whose square overflows has an
+    // infinite change, which the stop test takes for divergence
+    static __device__ __forceinline__ R rcp(R x) { return 1.0 / x; }
+    static __device__ __forceinline__ R fsqrt(R x) { return sqrt(x); }
     // constants of a cavity in R, and the wall mirror constants in S
     static __device__ __forceinline__ R dt(const CavityDesc* d) { return d->dt; }
     static __device__ __forceinline__ R beta_g(const CavityDesc* d) { return d->beta_g; }
