@@ -86,8 +86,7 @@ struct Desc3 {
 using rtlbfs::CavityCtl;
 using rtlbfs::CavityRun;
 
-// Constants of a mesh in the arithmetic type R and mirror constants in the
-// storage type S of a policy.
+// Constants of a mesh, FP64 (the FP32 kernel reads the f_ fields in place).
 template <class P>
 struct Cst;
 template <>
@@ -98,15 +97,6 @@ struct Cst<StoreD> {
     static __device__ __forceinline__ double force(const Desc3& d, int a) { return d.force[a]; }
     static __device__ __forceinline__ double uw(const Desc3& d, int s, int c) { return d.bcU[s][c]; }
     static __device__ __forceinline__ double Tw(const Desc3& d, int s) { return d.bcT[s]; }
-};
-template <>
-struct Cst<StoreQ> {
-    static __device__ __forceinline__ float beta_g(const Desc3& d) { return d.f_beta_g; }
-    static __device__ __forceinline__ float T_ref(const Desc3& d) { return d.f_T_ref; }
-    static __device__ __forceinline__ float dt(const Desc3& d) { return d.f_dt; }
-    static __device__ __forceinline__ float force(const Desc3& d, int a) { return d.f_force[a]; }
-    static __device__ __forceinline__ float uw(const Desc3& d, int s, int c) { return d.f_bcU[s][c]; }
-    static __device__ __forceinline__ float Tw(const Desc3& d, int s) { return d.f_bcT[s]; }
 };
 
 // Source index of coordinate c on an axis of n cells: wrap when periodic;

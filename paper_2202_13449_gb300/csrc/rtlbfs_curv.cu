@@ -168,12 +168,7 @@ struct CstC<StoreD> {
     static __device__ __forceinline__ double inf(const DescC& d, int q) { return d.d_inf[q]; }
 };
 template <>
-struct CstC<StoreQ> {
-    static __device__ __forceinline__ float gdir(const DescC& d, int a) { return d.f_gdir[a]; }
-    static __device__ __forceinline__ float force(const DescC& d, int a) { return d.f_force[a]; }
-    static __device__ __forceinline__ float beta_g(const DescC& d) { return d.f_beta_g; }
-    static __device__ __forceinline__ float T_ref(const DescC& d) { return d.f_T_ref; }
-    static __device__ __forceinline__ float dt(const DescC& d) { return d.f_dt; }
+struct CstC<StoreQ> {  // the ghost rules' (the FP32 kernel reads the others in place)
     static __device__ __forceinline__ float uw(const DescC& d, int s, int c) { return d.f_bcU[s][c]; }
     static __device__ __forceinline__ float Tw(const DescC& d, int s) { return d.f_bcT[s]; }
     static __device__ __forceinline__ float inf(const DescC& d, int q) { return d.f_inf[q]; }

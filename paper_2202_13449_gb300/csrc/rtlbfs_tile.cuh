@@ -31,7 +31,7 @@ struct TileSmem {
     FaceLine<R> yl[TY + 1];
     CellLine<R> xc[BX];
     CellLine<R> yc[BY];
-    R red[NT < 32 ? 1 : NT / 32][4];  // per-warp residual partials (tile_sums adds them)
+    R red[NT / 32][4];  // per-warp residual partials (tile_sums adds them)
     CavityDesc desc;  // the tile's cavity, staged by stage_tile
     int plan[3];      // the tile's step after its cavity's stop test: done, cur, sum slot
     int last;         // persistent kernel: this block finalises the step
