@@ -200,6 +200,7 @@ STEP3_SOURCES = ["paper_2202_13449_gb300/csrc/rtlbfs3d.cu",
                  "paper_2202_13449_gb300/csrc/rtlbfs3d_dev.cuh",
                  "paper_2202_13449_gb300/csrc/rtlbfs3d_pair.cuh",
                  "paper_2202_13449_gb300/csrc/rtlbfs_pair.cuh",
+                 "paper_2202_13449_gb300/csrc/rtlbfs_smem.h",
                  "paper_2202_13449_gb300/csrc/rtlbfs_dev.cuh"]
 CURV_SOURCES = ["paper_2202_13449_gb300/csrc/rtlbfs_curv.cu",
                 "paper_2202_13449_gb300/csrc/rtlbfs_curv_pair.cuh",
@@ -208,6 +209,7 @@ CURV_SOURCES = ["paper_2202_13449_gb300/csrc/rtlbfs_curv.cu",
 STEP_SOURCES = ["paper_2202_13449_gb300/csrc/rtlbfs_step.cu",
                 "paper_2202_13449_gb300/csrc/rtlbfs_march.cu",
                 "paper_2202_13449_gb300/csrc/rtlbfs_march2.cu",
+                "paper_2202_13449_gb300/csrc/rtlbfs_smem.h",
                 "paper_2202_13449_gb300/csrc/rtlbfs_pair.cuh",
                 "paper_2202_13449_gb300/csrc/rtlbfs_tile_pair.cuh",
                 "paper_2202_13449_gb300/csrc/rtlbfs_dev.cuh",

@@ -461,13 +461,14 @@ step3_kernel(const Desc3* __restrict__ dp, CavityRun* __restrict__ run, int par)
         // x- and y-faces of plane k.  The second, mostly empty rounds of the
         // x-faces, the y-faces and the gradients start on warps 0, 1 and 2: an
         // FP64 instruction costs the same with one lane or 32, and a block waits
-        // for its slowest warp (all three on warp 0: 80^3 1337 us, now 1253).
+        // for its slowest warp (two loops in 16 x 8 tiles, all three on warp 0:
+        // 80^3 1357 us; so: 1273).
         const int vs = mod3(k), gs = mod2(k);
         constexpr int NXF = TY * (TX + 1), NYF = (TY + 1) * TX;
         // 16 x 8: one loop over both kinds (face t < NXF an x-face) takes 9
-        // warp rounds instead of 5 + 5: 80^3 1253 -> 1199 us, TLBFS 2037 ->
-        // 1903.  Where it saves no round the two loops are 1-2 % faster
-        // (32 x 4 1442 against 1472 us).
+        // warp rounds instead of 5 + 5: 80^3 1273 -> 1217 us, TLBFS 2034 ->
+        // 1915.  Where it saves no round the two loops are 1-2 % faster
+        // (32 x 4 1464 against 1475 us, 32 x 8 1430 against 1446).
         constexpr bool ONE = (NXF + NYF + 31) / 32 < (NXF + 31) / 32 + (NYF + 31) / 32;
         if constexpr (ONE) {
             for (int t = tid; t < NXF + NYF; t += NT) {
@@ -924,7 +925,7 @@ int resolve(rtlbfs3d_ctx* h)
 // (latency hides in the others' gaps), in FP64 by the share of the FP64 units
 // each needs.  80^3 in 16 x 8 tiles, time over that of the pick, modelled and
 // measured: FP32 (pick 7 planes, 48 us) 4 planes 1.22 and 1.26, 8 planes 1.11
-// and 1.11; FP64 (pick 14, 1206 us) 4 planes 1.13 and 1.09, 8 planes 1.18 and
+// and 1.11; FP64 (pick 14, 1217 us) 4 planes 1.13 and 1.09, 8 planes 1.18 and
 // 1.15.  Where the mesh leaves SMs idle the pick is a plane or two: 16^3 12 us
 // (FP64 83), against 22 (236) with chunks of 4.
 double model_step(const rtlbfs3d_ctx* h, int tile, int& kc)

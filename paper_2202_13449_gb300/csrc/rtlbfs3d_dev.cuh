@@ -60,7 +60,8 @@ struct CellNT3 {
 // the same numbers with a third fewer operations (281 a face against 435
 // for products at the 19 nodes), and without the cancellation of the node
 // differences.  FP64 runs at the FMA rate, so there the step follows the
-// count: 20 steps of an 80^3 mesh and the download, FP64, 34.8 -> 29.0 ms.
+// count: 20 steps of an 80^3 mesh and the download, FP64, 34.8 -> 29.5 ms with
+// the step kernel of that time.
 //
 // The first stage, face3_columns, forms the coefficients C, S1, S2 of the
 // five primitives on the three columns (A: a = -1, M: a = 0, B: a = +1);

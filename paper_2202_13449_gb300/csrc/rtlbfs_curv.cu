@@ -415,8 +415,8 @@ __global__ void __launch_bounds__(TX* TY) curv_step_kernel(const DescC* __restri
 
     // 2. gradients on the tile and a 1-cell ring
     // (second rounds of gradients, i- and j-faces on warps 2, 0 and 1: a block
-    // waits for its slowest warp.  FP64 450 x 300 204.6 -> 200.0 us, 150 x 100
-    // 64.9 -> 57.8)
+    // waits for its slowest warp.  FP64 450 x 300 206.7 us with all on warp 0,
+    // 202.2 so; 150 x 100 64.2 and 56.9)
     for (int t = (tid + NT - 64) % NT; t < GX * GY; t += NT) {
         const int r = t / GX + 1, c = t % GX + 1;
         int is, xs, js, ys;

@@ -2,10 +2,10 @@
 // adjacent along i (included by rtlbfs_curv.cu; FP64: curv_step_kernel there).
 //
 // The phases of curv_step_kernel on the same tiles, one thread per pair of
-// cells.A thread per cell in scalar arithmetic,
-// with the geometry as records, ran 1980 instructions a cell; this runs 1000
-// (its share of the copies, loads and ghost items included).  Steps of
-// 300 x 200, 450 x 300 and 1800 x 1200 cells: 6.6, 9.3 and 123 us, before 8.35, 11.4 and 164.
+// cells.  A thread per cell in scalar arithmetic, with the geometry as records,
+// ran 1980 instructions a cell; this runs 1000 (its share of the copies, loads
+// and ghost items included).  Steps of 300 x 200, 450 x 300 and 1800 x 1200
+// cells: 6.6, 9.1 and 120 us, before 8.35, 11.4 and 161.
 // Small meshes are bound by the chain of latencies from one launch to the
 // next (5.6 us at 150 x 100), large ones by how many warps the 46 KB of staged
 // geometry per block let wait for shared memory: 2.8 TB/s and half of the

@@ -150,9 +150,10 @@ __host__ __device__ inline double r12(double num, double den)
 
 // The two words of a double, and tests on them.  The stop test stands at the
 // head of every step kernel's chain, and an FP64 operation there takes about
-// as long as twenty integer ones (an FP64 comparison too).  With the sums of
-// warp_sum4 and add_sums below: 512^2 10.95 -> 10.40 us per step, 1024x512
-// 21.6 -> 19.2, 301x203 6.75 -> 6.30, 64^2 6.5 -> 5.95.
+// as long as twenty integer ones (an FP64 comparison too).  With FP64
+// comparisons here and twenty shuffles in place of warp_sum4's six, a step of
+// 512^2 takes 10.88 us instead of 10.57, 301x203 5.83 instead of 5.53, 64^2 3.76
+// instead of 3.48, 400^2 in FP64 188 instead of 183.
 __host__ __device__ inline unsigned hi_word(double x)
 {
 #ifdef __CUDA_ARCH__
@@ -388,8 +389,9 @@ struct CellNT {
 // chain from the negated left column), and the middle column's slopes enter
 // doubled (D = 2 s_0 = s_-1 + s_+1), the powers of two going into constants:
 // 153 operations a face where forming each term by itself takes 172.  (In
-// FP64 the step runs at the FMA rate: 40 steps of a 400^2 mesh 8.44 -> 8.15 ms;
-// FP32 512^2 11.46 -> 11.26 ms for 1000 steps.)
+// FP64 the step runs at the FMA rate.  The first 16 of the 19, in the kernels of
+// that time: 40 steps of a 400^2 mesh 8.44 -> 8.15 ms; FP32 512^2 11.46 -> 11.26
+// ms for 1000 steps.)
 //
 // The first stage, face_columns, forms the column coefficients: values A, M,
 // B of the four primitives on a = -1, 0, +1, the negated slopes Na on a =
@@ -534,7 +536,7 @@ __host__ __device__ __forceinline__ void face_flux(const CellNT<V>& L, const Cel
 // u_t and rho u_n T exactly, so only the nodes' equilibria are formed one by
 // one, without their weights, and summed by weight and sign: 230 operations
 // a face where the equilibria of both states take 330 (512^2 FP32 14.7 -> 12.7 us
-// per step, FP64 492 -> 368).
+// per step, FP64 492 -> 358, with the tile of pairs and two FP64 blocks an SM).
 template <typename V, class W>
 __host__ __device__ __forceinline__ void face_flux_tlbfs_wall(const CellNT<V>& L, const CellNT<V>& Rc,
                                                              V Tbar, const FaceLine<V>& fl, W wall,

@@ -647,7 +647,7 @@ int Engine::set_chunk_rows(int rows)
 // tiles for their smaller halo.
 // FP64 is bound by its narrow units, for which every warp instruction counts
 // the same however few lanes it serves: a tile's FP64 warp instructions
-// (rounds of faces 175, of gradients 32, of updates 170).
+// (rounds of faces about 175, of gradients 32, of updates 170).
 int Engine::pick_tile_height(double* us) const
 {
     if (scheme_ == kSchemeTLBFS) return kTileYDefault;
@@ -727,9 +727,10 @@ int Engine::rebuild_tiles()
     // A single cavity, unless a schedule was set: FP32 marches where that is modelled faster
     // (from about 1 M cells: 1024^2 33.4, 2048^2 99.5 us per step
     // against the tiles' 35.3 and 133; 700^2 20.4 against 18.8), FP64 takes tiles
-    // (64^2: 17 us against 269 in 16-row chunks, a serial chain of 20 rows).
+    // (64^2: 17.5 us against 260 in 16-row chunks, a serial chain of 20 rows).
     // A batch marches: its cavities come and go, and a kernel that followed
-    // the mix would change a cavity's rounding on the way.
+    // the mix would change a cavity's rounding on the way.  (So can the rows of
+    // a unit, by the temperature that a unit's values are taken relative to.)
     if (auto_kernel_) {
         double tile_us = 0.0, march_us = 0.0;
         if (precision_ == RTLBFS_FP32) {

@@ -13,8 +13,9 @@
 //   the y-faces between rows j and j+1 (all in the lane's registers),
 //   the update of row j (the second cell's east face is lane l+1's first)
 //     and the residual sums.
-// No shared memory, no block barriers; every face is computed once (plus the
-// strip-edge halo); HBM sees one read and one write of the state per cell.
+// No block barriers; shared memory holds only what a lane reads back itself (a
+// ring of raw rows, the x-face constants); every face is computed once (plus
+// the strip-edge halo); HBM sees one read and one write of the state per cell.
 //
 // Why two columns a lane: the step is bound by instruction issue and the FMA
 // pipe.  A packed instruction does two columns' operation in one issue slot;

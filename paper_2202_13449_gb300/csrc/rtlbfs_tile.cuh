@@ -561,8 +561,9 @@ __device__ __forceinline__ void tile_step(TileSmem<P, TX, TY, NT>& sm, int i0, i
 // sub-partition, share a tile of 32 cells: every gradient (72) and every
 // face (82, x- and y-faces in one loop) gets a thread of its own, and in the
 // update warp k advances component k of all cells and then adds up one of
-// the residual sums: a chain of about 32 + 165 + 55 instructions, where the
-// 32 x 4 tile's warps pass through some 750.  64^2: 29.4 -> 17.6 us per step.
+// the residual sums: one gradient, one face and a part of an update, where the
+// 32 x 4 tile's warps pass through some 750 FP64 instructions.  64^2: 17.5 us per
+// step, in 32 x 4 tiles 27.5.
 template <class P, int TX, int TY, int NT, bool LDCG>
 __device__ __forceinline__ void tile_step_flat(TileSmem<P, TX, TY, NT>& sm, int i0, int j0,
                                                const Vec4<typename P::S>* __restrict__ fin,
@@ -727,8 +728,8 @@ namespace rtlbfs {
 // Resident blocks per SM to compile for: FP32 as many as the tile buffers
 // allow with some 96 registers a thread (wide blocks: two, then one); FP64
 // takes the registers it needs, but no more than let two of its large blocks
-// share an SM (512^2 in 8-row tiles: 279 us per step at 130 registers, 254 at
-// 128).
+// share an SM (512^2 in 8-row tiles: 295 us per step without the bound, 255 with
+// it; TLBFS 375 and 358; 400^2 182 and 183).
 template <class P, int TX, int TY, int NT>
 struct MinBlocks {
     static constexpr int value = NT == 256 ? 2 : 1;

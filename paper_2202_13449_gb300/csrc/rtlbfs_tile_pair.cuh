@@ -10,7 +10,7 @@
 //   - ghost columns hold mirrored values two deep, so gradients need no rule
 //     for them, and mirror rules are selected, not branched to;
 //   - the descriptor is read from shared memory.
-// 64^2 5.95 -> 3.35 us per step, 128^2 6.3 -> 3.7, 301x203 6.30 -> 5.45,
+// 64^2 5.95 -> 3.45 us per step, 128^2 6.3 -> 3.7, 301x203 6.30 -> 5.5,
 // 1024x512 19.2 -> 18.7, 512^2 10.4 -> 10.5 (bound by the launch and the
 // barriers of four blocks in step); TLBFS 512^2 14.7 -> 12.7.
 #pragma once
