@@ -7,8 +7,8 @@
 // and update arithmetic runs two cells an instruction.  80^3 in 16 x 8 tiles:
 // 48 us a step; a thread per cell in scalar arithmetic took 67, issue-bound at
 // 3250 instructions a cell.  What bounds it now is latency: 1500 instructions
-// a cell keep the schedulers busy a third of the time with the 8 warps that
-// 230 registers a thread leave room for (large meshes in 32 x 8: half of it with 12).
+// a cell keep the schedulers busy 40 % of the time with the 8 warps that 234
+// registers a thread leave room for (large meshes in 32 x 8: half of it with 12).
 //  - Face fluxes change hands as registers (x: shuffles) or through shared
 //    memory (y, and the tile's east column), so that three 32 x 8 blocks fit.
 //  - Raw records of the plane to come are fetched after the faces, which need

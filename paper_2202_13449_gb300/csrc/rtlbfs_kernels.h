@@ -9,11 +9,11 @@
 namespace rtlbfs {
 
 // Tiles of the shared-memory step kernel: kTileX = 32 columns (16 for the
-// 2-row FP64 tile, see tile_width) by one of the compiled heights below, 16
-// threads per tile row (two cells per thread in the update).  The height is picked per cavity set so that the number of
-// tiles fills the SMs evenly (a 512-row mesh in 16-row tiles leaves a third
-// of the SMs one tile short); the low heights spread small meshes over many
-// SMs, which matters most in FP64, where an SM does 2 FMAs per clock.
+// 2-row FP64 tile, see tile_width) by one of the compiled heights below.  The
+// height is picked per cavity set so that the number of tiles fills the SMs
+// evenly (a 512-row mesh in 16-row tiles leaves a third of the SMs one tile
+// short); the low heights spread small meshes over many SMs, which matters
+// most in FP64, where an SM does 2 FMAs per clock.
 constexpr int kTileX = 32;
 constexpr int kTileHeights[] = {16, 14, 12, 10, 8, 4, 2};
 constexpr int kTileYDefault = 16;

@@ -1,6 +1,6 @@
 // rtlbfs_persist.cu -- the tile step of rtlbfs_step.cu in persistent form:
 // one launch advances one cavity by many explicit time steps (arXiv
-// 2202.13449, Section 3.2), with the same arithmetic (tile_step) and the
+// 2202.13449, Section 3.2), with the same arithmetic (run_tile) and the
 // same stop test after every step.
 //
 // Launch: cooperative, one block per tile, every tile resident at once.

@@ -1,8 +1,9 @@
 // rtlbfs_tile.cuh -- one tile of the fused RTLBFS time step (arXiv
 // 2202.13449, Section 3.2) on a structured 2D mesh: the shared-memory tile
 // buffers, ghost resolution and mirror rules, Green-Gauss gradients and the
-// tile_step() body shared by the launch-per-step tile kernel
-// (rtlbfs_step.cu) and the persistent tile kernel (rtlbfs_persist.cu).
+// run_tile() body shared by the launch-per-step tile kernel (rtlbfs_step.cu)
+// and the persistent tile kernel (rtlbfs_persist.cu): tile_step and
+// tile_step_flat in FP64, tile_step_pair (rtlbfs_tile_pair.cuh) in FP32.
 #pragma once
 
 #include <cuda_runtime.h>
